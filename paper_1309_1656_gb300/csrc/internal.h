@@ -116,6 +116,10 @@ const LatticeOps *ops_d2q9_fp64df();
 const LatticeOps *ops_d3q19_fp64df();
 // the double-float step on FP64 storage (kernels_<lattice>_fp64df.cu)
 template <int D> cudaError_t step_f64df(qlbm_ctx *h, bool odd);
+// The FP64 step on the integer pipes (kernels_<lattice>_fp64_fix.cu): mode 0
+// even AA step, 1 odd, 2 two-buffer step from src to dst.  False, with nothing
+// launched, where it does not apply (a magnetic field; omega > 2).
+template <int D> bool step_fix(qlbm_ctx *h, int mode, const void *src, void *dst, cudaError_t *err);
 
 inline const LatticeOps *lattice_ops(int d, int prec)
 {

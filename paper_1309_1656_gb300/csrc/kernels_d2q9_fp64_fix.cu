@@ -1,0 +1,28 @@
+// D2Q9 kernels of the FP64 step on the integer pipes (fix64.cuh): the AA
+// steps and the two-buffer step of the reverse mode, compiled apart from the
+// rest of the FP64 dispatch table.
+#include "fix64.cuh"
+#include "launch.cuh"
+
+namespace qlbm {
+
+template <int D> bool step_fix(qlbm_ctx *h, int mode, const void *src, void *dst, cudaError_t *err)
+{
+    FixConst fc;
+    if (h->mag != FIELD_NONE || !make_fix_const(h->hc, h->dt / h->tau, &fc)) return false;
+    using L = Launchers<D, CodecF64>;
+    const Chunks ch = make_chunks(h->g);
+    const Planes<double, Lattice<D>::Q> s = L::template planes_of<double>(h, src), d = L::template planes_of<double>(h, dst);
+    const Coll<double> k = make_coll<double>(h);
+    const dim3 blk(kFixBlock), grd((unsigned)((ch.total + kFixBlock / 32 - 1) / (kFixBlock / 32)));
+    switch (mode) {
+    case FIX_EVEN: k_step_fix<D, FIX_EVEN><<<grd, blk, 0, h->stream>>>(s, d, h->g, fc, k, ch, h->flags); break;
+    case FIX_ODD: k_step_fix<D, FIX_ODD><<<grd, blk, 0, h->stream>>>(s, d, h->g, fc, k, ch, h->flags); break;
+    default: k_step_fix<D, FIX_PUSH><<<grd, blk, 0, h->stream>>>(s, d, h->g, fc, k, ch, h->flags); break;
+    }
+    *err = cudaGetLastError();
+    return true;
+}
+template bool step_fix<2>(qlbm_ctx *, int, const void *, void *, cudaError_t *);
+
+}  // namespace qlbm

@@ -195,6 +195,11 @@ template <int D, class Codec> struct Launchers {
 
     static cudaError_t push(qlbm_ctx *h, const void *src, void *dst)
     {
+        if constexpr (std::is_same<Codec, CodecF64>::value) {
+            // the arithmetic of the step it stands for, bit for bit
+            cudaError_t e;
+            if (step_fix<D>(h, 2, src, dst, &e)) return e;
+        }
         const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
         return with_field(h->mag, [&](auto fc) {
             constexpr int F = decltype(fc)::value;

@@ -13,6 +13,10 @@ namespace qlbm {
 template <int D, class Codec>
 cudaError_t Launchers<D, Codec>::step(qlbm_ctx *h, bool odd)
 {
+    if constexpr (std::is_same<Codec, CodecF64>::value) {
+        cudaError_t e;
+        if (step_fix<D>(h, odd ? 1 : 0, h->pop, h->pop, &e)) return e;
+    }
     const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
     const Planes<S, Q> pl = planes(h);
     const Coll<R> k = make_coll<R>(h);
