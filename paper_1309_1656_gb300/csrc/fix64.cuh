@@ -1,14 +1,13 @@
 // The FP64 step on the integer pipes (QLBM_FP64 storage, no field).
 //
-// GB300's double-precision pipe takes 64 issue cycles per warp instruction
-// (measured: one DFMA per 64.0 cycles and sub-partition, whatever the number
-// of warps; integer add, logic and minimum 1, shifts and 32-bit multiplies 2,
-// the 32x32->64 multiply 4).  The step of k_step_aa<D, CodecF64> is bound by
-// that pipe alone: ~445 double-precision instructions per D3Q19 site, at
-// 128^3 1485 us for 2.55 GB that the copy rate moves in 376 us.  This file
-// does the same step (Eqs. DiscrAvr, WeqAlgo, CollisionStep, TransportStep)
-// without one double-precision instruction, in fixed point with more digits
-// than a double has:
+// GB300's double-precision pipe takes 64 cycles per warp instruction and
+// sub-partition (measured, whatever the number of warps; integer add, logic
+// and minimum take 1, shifts and 32-bit multiplies 2, the 32 x 32 -> 64-bit
+// multiply 4).  The step of k_step_aa<D, CodecF64> is bound by that pipe
+// alone: ~445 double-precision instructions per D3Q19 site, at 128^3 1485 us
+// for 2.55 GB that the copy rate moves in 376 us.  This file does the same
+// step (Eqs. DiscrAvr, WeqAlgo, CollisionStep, TransportStep) in fixed point
+// with more digits than a double has:
 //
 //   * a component's b values at a site are aligned to their largest one's
 //     exponent: X = v / U as 64-bit integers with |X| < 2^58 (a double up to
@@ -18,26 +17,32 @@
 //     ratios J/n and E2/n with 2^-60 steps, as sums of ten basis values
 //     (class constants, i.j and its products), and
 //       W_i' = (1 - omega) W_i + h_i M,   M = sum_j W_j of the component,
-//     is one pair of 64 x 64-bit products whose 96 leading bits are kept;
-//   * the result is normalised and rounded once to a double.
+//     is a pair of 64 x 64-bit products, rounded to 2^-56 of the largest;
+//   * one conversion per value rounds it to a double (the only use of the
+//     double pipe, which runs beside the integer ones).
 //
-// Measured: D3Q19 128^3 1484 -> 835 us (even step), 2048 x 2 D2Q9 9.2 -> 4.1 us.
-//
-// Each step above errs by at most ~2^-57 of the component's largest value at
-// the site, the result by its own rounding besides; the double-precision step
-// rounds h, h M - W and W' (tests/test_gpu_fix64.py compares both with the
-// 64-bit oracle).  Sites outside the fixed-point form's range (non-finite
-// or extreme values, n <= 0, |j| >= 1/2, |h| >= 1) are stepped in double by
-// their warp, with the same flags as k_step_aa.
+// Each result errs by at most ~1.2 x 2^-53 of its component's largest value
+// at the site (0.13 rms; the double-precision step, which rounds h, h M - W
+// and W', by up to 8 x 2^-53, 0.5 rms, at omega = 0.5, and more above).
+// Warps with a site outside the form's range (non-finite or extreme values,
+// n <= 0, |j| >= 3/8, E2/n a unit off, |h| >= 1) step in double, with the same
+// flags as k_step_aa.
 //
 // Layout: four lanes per site, lane c holding component c (f, s_x, s_y, s_z)
 // of its b populations.  A site's vector of four doubles is 32 bytes, so a
 // warp's 8-byte accesses cover 256 consecutive bytes (8 sites), every value
-// is read and written once, and a thread keeps 19 values instead of 76 (20
-// resident warps per SM instead of 8).
+// is read and written once, and a thread keeps 19 values instead of 76.
+// Blocks of two warps (a 64 x 64 lattice reaches every SM); 16 warps per SM
+// at 128 registers for D3Q19 (20 at 96 spill: 548 us).
+//
+// Measured (double-precision kernel -> this one): D3Q19 128^3 1485 -> 507 us,
+// D2Q9 2048^2 1512 -> 527 us, D2Q9 64^2 8.3 -> 2.65 us and 2048 x 2 9.2 -> 2.7
+// us per step.  Now bound by issue and the integer and multiply pipes
+// together (60-64 % each, ~1390 instructions per warp of 8 sites).
 #pragma once
 
 #include <math.h>
+#include <string.h>
 
 #include "internal.h"
 #include "step.cuh"
@@ -45,16 +50,21 @@
 namespace qlbm {
 
 #ifdef __CUDA_ARCH__
-__device__ __forceinline__ long long fx_mulhi(long long a, long long b) { return __mul64hi(a, b); }
-__device__ __forceinline__ unsigned long long fx_umulhi(unsigned long long a, unsigned long long b)
+// a b + c, and a b: one multiply-add each (written out: from the C expression
+// the compiler adds separately, 22 instructions more per updated value)
+__device__ __forceinline__ long long fx_mad(int a, int b, long long c)
 {
-    return __umul64hi(a, b);
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
 }
-__device__ __forceinline__ int fx_mulhi32(int a, int b) { return __mulhi(a, b); }
+__device__ __forceinline__ unsigned long long fx_umad(unsigned a, unsigned b, unsigned long long c)
+{
+    unsigned long long r;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
 __device__ __forceinline__ int fx_clz(unsigned a) { return __clz((int)a); }
-__device__ __forceinline__ int fx_clz64(unsigned long long a) { return __clzll((long long)a); }
-__device__ __forceinline__ unsigned fx_shf_l(unsigned lo, unsigned hi, int s) { return __funnelshift_l(lo, hi, s); }
-__device__ __forceinline__ unsigned fx_shf_r(unsigned lo, unsigned hi, int s) { return __funnelshift_r(lo, hi, s); }
 // v >> s for any s >= 0 (0 from 64 on)
 __device__ __forceinline__ unsigned long long fx_shr(unsigned long long v, int s)
 {
@@ -62,46 +72,67 @@ __device__ __forceinline__ unsigned long long fx_shr(unsigned long long v, int s
     asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(s));
     return r;
 }
-__device__ __forceinline__ float fx_rcp(float x) { return __frcp_rn(x); }
+// 1/x to ~1 ulp
+__device__ __forceinline__ float fx_rcp(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float fx_float(unsigned b) { return __uint_as_float(b); }
+__device__ __forceinline__ unsigned fx_bits(float v) { return __float_as_uint(v); }
 #else   // the same functions for the host (arithmetic checks without a GPU)
-inline long long fx_mulhi(long long a, long long b) { return (long long)(((__int128)a * b) >> 64); }
-inline unsigned long long fx_umulhi(unsigned long long a, unsigned long long b)
+inline long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
+inline unsigned long long fx_umad(unsigned a, unsigned b, unsigned long long c)
 {
-    return (unsigned long long)(((unsigned __int128)a * b) >> 64);
+    return (unsigned long long)a * b + c;
 }
-inline int fx_mulhi32(int a, int b) { return (int)(((long long)a * b) >> 32); }
 inline int fx_clz(unsigned a) { return a ? __builtin_clz(a) : 32; }
-inline int fx_clz64(unsigned long long a) { return a ? __builtin_clzll(a) : 64; }
-inline unsigned fx_shf_l(unsigned lo, unsigned hi, int s)
-{
-    s &= 31;
-    return s ? (hi << s) | (lo >> (32 - s)) : hi;
-}
-inline unsigned fx_shf_r(unsigned lo, unsigned hi, int s)
-{
-    s &= 31;
-    return s ? (lo >> s) | (hi << (32 - s)) : lo;
-}
 inline unsigned long long fx_shr(unsigned long long v, int s) { return s > 63 ? 0 : v >> s; }
 inline float fx_rcp(float x) { return 1.0f / x; }
+inline float fx_float(unsigned b)
+{
+    float v;
+    memcpy(&v, &b, 4);
+    return v;
+}
+inline unsigned fx_bits(float v)
+{
+    unsigned b;
+    memcpy(&b, &v, 4);
+    return b;
+}
 #endif
 
 #define FX_FN __host__ __device__ __forceinline__
 
+// v = hi 2^32 + lo with lo signed: products of two splits then need signed
+// 32 x 32 -> 64-bit multiply-adds only.
+struct FxSplit {
+    int hi, lo;
+};
+FX_FN FxSplit fx_split(long long v)
+{
+    FxSplit r;
+    r.lo = (int)v;
+    r.hi = (int)(v >> 32) + (int)((unsigned)r.lo >> 31);
+    return r;
+}
 // Constants of the fixed-point step, "qN" meaning the value times 2^N:
 //   h_i of class m = |i|^2:  h = al[m] + be[m] d + ga[m] |j|^2 + (linear and
-//   quadratic terms in i.j),  d = E2/n - |j|^2,
-//   al = omega w (1 - (m K - c) c inv),  be = omega w (m K - c) K inv,
-//   ga = omega w c5,  inv = 1/(m4 - c^2)  (P_i of Eq. WeqAlgo with alpha1 and
-//   alpha2 written out), and for the axis class c3 = omega w_1 c3,
-//   c4 = omega w_1 c4; the diagonal class has w_2 = w_1 / 2 (D3Q19) or
-//   w_1 / 4 (D2Q9) exactly, so its terms are shifts of these.
+//   quadratic terms in i.j),  d = E2/n - |j|^2 - d0,  d0 = c/K,
+//   al = omega w,  be = omega w (m K - c) K / (m4 - c^2),  ga = omega w c5
+// (P_i of Eq. WeqAlgo with alpha1 and alpha2 written out: alpha2 is
+// K d / (m4 - c^2)), and for the axis class c3 = omega w_1 c3, c4 = omega w_1
+// c4; the diagonal class has w_2 = w_1 / 2 (D3Q19) or w_1 / 4 (D2Q9) exactly,
+// so its terms are shifts of these.
 struct FixConst {
-    long long omc;          // q62: 1 - omega
-    long long al[3], be[3]; // q62
-    long long ga[2];        // q62, rest and axis class
-    long long c4;           // q62
-    long long c3;           // q63
+    FxSplit omc;            // q62: 1 - omega
+    long long al[3];        // q62
+    FxSplit be[3];          // q62
+    FxSplit ga[2];          // q62, rest and axis class
+    FxSplit c3, c4;         // q62
+    long long d0;           // q60
 };
 constexpr long long kFxOne = 1LL << 62;   // 1.0 in q62
 
@@ -122,70 +153,57 @@ FX_FN long long fx_align(unsigned hi, unsigned lo, int eb)
     return (x ^ s) - s;
 }
 
-// v = hi 2^32 + lo with lo signed.
-struct FxSplit {
-    int hi, lo;
-};
-FX_FN FxSplit fx_split(long long v)
+FX_FN long long fx_wide(int a, int b) { return (long long)a * b; }
+// a b / 2^64 without the product of the low words (at most a quarter of the
+// last place): qA x qB -> q(A + B - 64).
+FX_FN long long fx_mul(FxSplit a, FxSplit b)
 {
-    FxSplit r;
-    r.lo = (int)v;
-    r.hi = (int)(v >> 32) - (r.lo >> 31);
-    return r;
+    return fx_mad(a.hi, b.hi, fx_mad(a.hi, b.lo, fx_wide(a.lo, b.hi)) >> 32);
 }
 
-// The value t 2^32 + f (t the 64 leading bits, units 2^(e0 - 1078)) rounded
-// to a double; e0 = 25 stands for a component that is zero throughout.
-FX_FN unsigned long long fx_to_double(long long t, unsigned f, int e0)
+// t (units 2^(eb - 1078)) rounded to a double: one conversion, which takes
+// the double pipe the step otherwise leaves idle (64 cycles against ~15
+// integer instructions), and the exponent moved by shift = (eb - 1078) << 20.
+FX_FN double fx_to_double(long long t, int shift)
 {
-    const unsigned s = (unsigned)(int)(t >> 63);
-    unsigned a1 = (unsigned)(t >> 32) ^ s, a0 = (unsigned)t ^ s, a = f ^ s;
-    int lz = fx_clz(a1), ex = e0;
-    if (a1 == 0u && e0 != 25) {     // below 2^-24 of the largest value, or cancelled
-        a1 = a0;
-        a0 = a;
-        a = 0u;
-        ex -= 32;
-        if (a1 == 0u) {
-            a1 = a0;
-            a0 = 0u;
-            ex -= 32;
-            if (a1 == 0u) return 0ull;
-        }
-        lz = fx_clz(a1);
-    }
-    const unsigned m1 = fx_shf_l(a0, a1, lz), m0 = fx_shf_l(a, a0, lz);
-    unsigned long long r = ((unsigned long long)(m1 >> 11) << 32) | fx_shf_r(m0, m1, 11);
-    r += (m0 >> 10) & 1u;
-    r += (unsigned long long)(unsigned)((ex + 7 - lz) << 20) << 32;
-    return r | ((unsigned long long)(s & 0x80000000u) << 32);
+    const double v = (double)t;
+#ifdef __CUDA_ARCH__
+    const int hi = __double2hiint(v);
+    return __hiloint2double(hi ? hi + shift : 0, __double2loint(v));
+#else
+    return ldexp(v, shift / (1 << 20));
+#endif
 }
 
-// omc X + h m as (t, f) of fx_to_double: units of 4 U, and the next 32 bits
-// (of the products of the low words their high words).  |omc|, |h| <= 2^62 and
-// |m| <= 19 * 2^58 keep the cross terms in 64 bits.
-FX_FN void fx_update(long long X, FxSplit omc, long long h, FxSplit m, long long &t, unsigned &f)
+// omc X + h m in units of 4 U, rounded to nearest but for the products of the
+// low words, which are left out (2^-58 of the largest value at most; they
+// would take 3 of 9 multiplications on the pipe that bounds the kernel).
+// |omc|, |h| <= 2^62 and |m| <= 19 * 2^58 keep the cross terms in 64 bits.
+FX_FN long long fx_update(long long X, FxSplit omc, long long h, FxSplit m)
 {
     const FxSplit x = fx_split(X), g = fx_split(h);
-    const long long cross = (long long)x.lo * omc.hi + (long long)x.hi * omc.lo + (long long)m.lo * g.hi +
-                            (long long)m.hi * g.lo + ((long long)fx_mulhi32(x.lo, omc.lo) + fx_mulhi32(m.lo, g.lo));
-    t = (long long)x.hi * omc.hi + (long long)m.hi * g.hi + (cross >> 32);
-    f = (unsigned)cross;
+    const long long cross =
+        fx_mad(m.hi, g.lo, fx_mad(m.lo, g.hi, fx_mad(x.hi, omc.lo, fx_mad(x.lo, omc.hi, 0x80000000LL))));
+    return fx_mad(m.hi, g.hi, fx_mad(x.hi, omc.hi, cross >> 32));
 }
 
-// 1/x in q61 for nn = x 2^64, x in [1/2, 1): a single-precision reciprocal
-// and two Newton steps r <- r + r (1 - x r) in integers.
+// 1/x in q62 for nn = x 2^64, x in [1/2, 1): a single-precision reciprocal
+// and two Newton steps r <- r + r (1 - x r) in integers, each product cut
+// below 2^-62.
 FX_FN long long fx_recip(unsigned long long nn)
 {
-    const float xf = (float)(unsigned)(nn >> 40) * 0x1p-24f;
-    const unsigned R0 = (unsigned)(fx_rcp(xf) * 1073741824.f);      // q30
     const unsigned nh = (unsigned)(nn >> 32), nl = (unsigned)nn;
-    const unsigned long long p = (unsigned long long)nh * R0 + (((unsigned long long)nl * R0) >> 32);   // q62: x r
+    // 24 leading bits of x as a float in [1/2, 1); its reciprocal in q30
+    const unsigned rb = fx_bits(fx_rcp(fx_float(0x3f000000u | ((nh >> 8) & 0x7fffffu))));
+    const unsigned R0 = ((rb < 0x3fffffffu ? rb : 0x3fffffffu) << 7 | 0x40000000u) & 0x7fffffffu;
+    const unsigned long long p = fx_umad(nh, R0, fx_umad(nl, R0, 0) >> 32);      // q62: x r
     const long long e0 = kFxOne - (long long)p;
-    const unsigned long long r1 =
-        ((unsigned long long)R0 << 32) + (unsigned long long)(((long long)R0 * (int)(e0 >> 10)) >> 20);  // q62
-    const long long e1 = kFxOne - (long long)fx_umulhi(nn, r1);
-    return (long long)((r1 + (unsigned long long)(((long long)(unsigned)(r1 >> 32) * e1) >> 30)) >> 1);
+    const long long r1 = ((long long)R0 << 32) + (fx_wide((int)R0, (int)(e0 >> 10)) >> 20);      // q62
+    const unsigned rh = (unsigned)((unsigned long long)r1 >> 32), rl = (unsigned)r1;
+    const unsigned long long x1 = fx_umad(nh, rh, fx_umad(nh, rl, 0) >> 32) + (fx_umad(nl, rh, 0) >> 32);
+    const int e1 = (int)(kFxOne - (long long)x1);       // < 2^20
+    const long long r = r1 + (fx_wide((int)(rh >> 1), e1) >> 29);
+    return r < 0 ? 0x7fffffffffffffffLL : r;            // x = 1/2
 }
 
 // h_i of all directions as ten basis values (q62).
@@ -196,67 +214,73 @@ struct FixCoef {
     long long qo[3];                // axis class: c4 j_a j_b, (a, b) = (0,1), (0,2), (1,2)
 };
 
-// From n, J, E2 (all in the same units); false outside the range of the form.
+// From n, J, E2 (all in the same units); false outside the range of the form
+// (decided on high words).
 template <int D> FX_FN bool fx_coefficients(long long n, const long long (&J)[3], long long E, const FixConst &k,
                                             FixCoef &c)
 {
-    bool ok = n > 0;
-    const long long half = n >> 1;
-#pragma unroll
-    for (int a = 0; a < D; ++a) ok = ok && J[a] < half && J[a] > -half;
-    ok = ok && E >= 0 && (E >> 1) < n - (n >> 4);
-    if (!ok) return false;
-    const int lz = fx_clz64((unsigned long long)n);     // >= 1
-    const long long r = fx_recip((unsigned long long)n << lz);
-    long long j[3];     // q60
-#pragma unroll
-    for (int a = 0; a < D; ++a) j[a] = fx_mulhi(J[a] << (lz - 1), r);
-    const long long e = fx_mulhi((E >> 1) << (lz - 1), r) << 3;     // q62
-    long long sq[3], jj = 0;                                        // q62
+    // |j_a| < 3/8 (so |j|^2 < 1/2), 0 <= E2/n < 2
+    const int nh = (int)(n >> 32), Eh = (int)(E >> 32), lim = (nh >> 2) + (nh >> 3);
+    auto mag = [](long long v) { return abs((int)(v >> 32)); };
+    bool ok = Eh >= 0 && (Eh >> 1) < nh && mag(J[0]) < lim && mag(J[1]) < lim;
+    if (D == 3) ok = ok && mag(J[2]) < lim;
+    const int lz = fx_clz((unsigned)nh);    // 1..31 where ok
+    const FxSplit r = fx_split(fx_recip((unsigned long long)n << lz));
+    FxSplit j[3];       // q64
+    long long jj = 0;   // q64
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        sq[a] = fx_mulhi(j[a] << 3, j[a] << 3);
-        jj += sq[a];
-        c.B[a] = fx_mulhi(k.c3, j[a] << 2) << 1;
-        c.qd[a] = fx_mulhi(k.c4, sq[a]) << 2;
+        j[a] = fx_split(fx_mul(fx_split(J[a] << lz), r) << 2);
+        c.B[a] = fx_mul(k.c3, j[a]);
+        const long long sq = fx_mul(j[a], j[a]);
+        jj += sq;
+        c.qd[a] = fx_mul(k.c4, fx_split(sq));
     }
-    c.qo[0] = fx_mulhi(k.c4, fx_mulhi(j[0] << 3, j[1] << 3)) << 2;
+    c.qo[0] = fx_mul(k.c4, fx_split(fx_mul(j[0], j[1])));
     if (D == 3) {
-        c.qo[1] = fx_mulhi(k.c4, fx_mulhi(j[0] << 3, j[2] << 3)) << 2;
-        c.qo[2] = fx_mulhi(k.c4, fx_mulhi(j[1] << 3, j[2] << 3)) << 2;
+        c.qo[1] = fx_mul(k.c4, fx_split(fx_mul(j[0], j[2])));
+        c.qo[2] = fx_mul(k.c4, fx_split(fx_mul(j[1], j[2])));
     }
-    const long long d = e - jj, g1 = fx_mulhi(k.ga[1], jj) << 2;
-    c.b0 = k.al[0] + ((fx_mulhi(k.be[0], d) + fx_mulhi(k.ga[0], jj)) << 2);
-    c.b1 = k.al[1] + (fx_mulhi(k.be[1], d) << 2) + g1;
-    c.b2 = k.al[2] + (fx_mulhi(k.be[2], d) << 2) + (g1 >> (D == 3 ? 1 : 2));
-    // |h_i| < 1 for every direction: axis 1/2 + 1/8 + 1/4, diagonal at most
-    // 1/4 + 1/8 + 1/8 + 1/4 (magnitudes by or-ing, exact for powers of two)
-    auto mag = [](long long v) { return v ^ (v >> 63); };
-    long long q = mag(c.qd[0]) | mag(c.qd[1]) | mag(c.qo[0]), B = mag(c.B[0]) | mag(c.B[1]);
-    if (D == 3) {
-        q |= mag(c.qd[2]) | mag(c.qo[1]) | mag(c.qo[2]);
-        B |= mag(c.B[2]);
-    }
-    return mag(c.b0) < kFxOne && mag(c.b1) < kFxOne / 2 && ((mag(c.b2) | B) < kFxOne / 4) && q < kFxOne / 8;
+    const long long d60 = fx_mul(fx_split((E >> 1) << (lz - 1)), r) - k.d0 - (jj >> 4);
+    ok = ok && mag(d60) < (1 << 28);
+    const FxSplit d = fx_split(d60 << 3), s = fx_split(jj);     // q63, q64
+    const long long g1 = fx_mul(k.ga[1], s);
+    c.b0 = k.al[0] + fx_mul(k.ga[0], s) + 2 * fx_mul(k.be[0], d);
+    c.b1 = k.al[1] + g1 + 2 * fx_mul(k.be[1], d);
+    c.b2 = k.al[2] + (g1 >> (D == 3 ? 1 : 2)) + 2 * fx_mul(k.be[2], d);
+    // |h_i| < 1 for every direction: the other terms are bounded by |j_a| <
+    // 3/8 (make_fix_const)
+    constexpr int q62 = 1 << 30;
+    return ok && mag(c.b0) < q62 && mag(c.b1) < q62 / 2 && mag(c.b2) < q62 / 4;
 }
 
-// h_q (q62) of direction q (compile-time after unrolling).
-template <int D> FX_FN long long fx_h(const FixCoef &c, int q)
+// Calls f(q, h_q) for every direction, h_q in q62: the terms are shared
+// within the pairs +-a and the quadruples +-a +-b.
+template <int D, class F> FX_FN void fx_each_h(const FixCoef &c, F &&f)
 {
-    const int ex = cx<D>(q), ey = cy<D>(q), ez = cz<D>(q), cls = cnorm2<D>(q);
-    constexpr int sh = D == 3 ? 1 : 2;      // w_2 = w_1 >> sh
-    if (cls == 0) return c.b0;
-    if (cls == 1) {
-        const int a = ex ? 0 : (ey ? 1 : 2);
+    constexpr int Q = Lattice<D>::Q, sh = D == 3 ? 1 : 2;       // w_2 = w_1 >> sh
+    f(Q / 2, c.b0);
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        const int q = direction_of<D>(a == 0, a == 1, a == 2);
         const long long A = c.b1 + c.qd[a];
-        return (ex + ey + ez > 0) ? A + c.B[a] : A - c.B[a];
+        f(q, A + c.B[a]);
+        f(Q - 1 - q, A - c.B[a]);
     }
-    const int a = ex ? 0 : 1, b = ez ? 2 : 1;
-    const int ea = a == 0 ? ex : ey, eb = b == 2 ? ez : ey;
-    const long long qo = c.qo[a + b - 1] >> (sh - 1);
-    const long long A = c.b2 + ((c.qd[a] + c.qd[b]) >> sh) + (ea * eb > 0 ? qo : -qo);
-    const long long L = (ea > 0 ? c.B[a] : -c.B[a]) + (eb > 0 ? c.B[b] : -c.B[b]);
-    return A + (L >> sh);
+#pragma unroll
+    for (int a = 0; a < D - 1; ++a)
+#pragma unroll
+        for (int b = a + 1; b < D; ++b) {
+            const long long A = c.b2 + ((c.qd[a] + c.qd[b]) >> sh), C = c.qo[a + b - 1] >> (sh - 1);
+            const long long S = (c.B[a] + c.B[b]) >> sh, T = (c.B[a] - c.B[b]) >> sh;
+            const long long P = A + C, M = A - C;
+            const int qp = direction_of<D>(a == 0, a == 1 || b == 1, b == 2);
+            const int qm = direction_of<D>(a == 0, a == 1 ? 1 : (b == 1 ? -1 : 0), b == 2 ? -1 : 0);
+            f(qp, P + S);
+            f(Q - 1 - qp, P - S);
+            f(qm, M + T);
+            f(Q - 1 - qm, M - T);
+        }
 }
 
 // Double-double arithmetic for the constants (host): rounding them to double
@@ -295,15 +319,22 @@ inline bool make_fix_const(const HostConsts &k, double omega, FixConst *o)
     };
     const double q62 = 4611686018427387904.0;
     const Dd K(k.K), c(k.c), inv = reciprocal(Dd(k.m) + -(c * c)), om(omega);
-    o->omc = kFxOne - (omega < 1.0 ? llrint(omega * q62) : 2 * llrint(omega * q62 * 0.5));
+    const long long omc = kFxOne - (omega < 1.0 ? llrint(omega * q62) : 2 * llrint(omega * q62 * 0.5));
+    o->omc = fx_split(omc);
     for (int m = 0; m < 3; ++m) {
-        const Dd ow = om * Dd(k.w[m]), t = Dd(m) * K + -c;
-        o->al[m] = fix(ow * (Dd(1.0) + -(t * c * inv)), q62, 1.99);
-        o->be[m] = fix(ow * t * K * inv, q62, 1.99);
-        if (m < 2) o->ga[m] = fix(ow * K * Dd(k.alpha5), q62, 1.99);
+        const Dd ow = om * Dd(k.w[m]);
+        o->al[m] = fix(ow, q62, 1.0);
+        o->be[m] = fx_split(fix(ow * (Dd(m) * K + -c) * K * inv, q62, 1.99));
+        if (m < 2) o->ga[m] = fx_split(fix(ow * K * Dd(k.alpha5), q62, 1.99));
     }
-    o->c4 = fix(om * Dd(k.w[1]) * Dd(4.0) * K * K * Dd(k.alpha4), q62, 1.99);
-    o->c3 = fix(om * Dd(k.w[1]) * Dd(2.0) * K * Dd(k.alpha3), 2.0 * q62, 0.99);
+    // with |j_a| < 3/8 and class constants below 1, 1/2 and 1/4, |h_i| < 1:
+    // B = c3 3/8 and q = c4 9/64 bound the linear and quadratic terms
+    const Dd c3 = om * Dd(k.w[1]) * Dd(2.0) * K * Dd(k.alpha3), c4 = om * Dd(k.w[1]) * Dd(4.0) * K * K * Dd(k.alpha4);
+    const double B = fabs(c3.h) * 0.375, q = fabs(c4.h) * 0.140625, half = k.d == 3 ? 0.5 : 0.25;
+    ok = ok && 0.5 + q + B < 0.99 && 0.25 + half * (2 * q + 2 * B) + 2 * half * q < 0.99;
+    o->c3 = fx_split(fix(c3, q62, 1.99));
+    o->c4 = fx_split(fix(c4, q62, 1.99));
+    o->d0 = fix(c * reciprocal(K), q62 / 4.0, 2.0);
     return ok;
 }
 
@@ -338,7 +369,7 @@ inline Chunks make_chunks(const Grid &g)
     c.y = make_fast_div((unsigned)g.ny);
     return c;
 }
-constexpr int kFixBlock = 128;
+constexpr int kFixBlock = 64;
 
 __device__ __forceinline__ long long fx_from_lane0(long long v)
 {
@@ -391,7 +422,7 @@ __device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[La
 // reverse mode (as k_step_push), with the same arithmetic in all three.
 enum : int { FIX_EVEN = 0, FIX_ODD = 1, FIX_PUSH = 2 };
 template <int D, int MODE>
-__global__ void __launch_bounds__(kFixBlock, D == 3 ? 5 : 8)
+__global__ void __launch_bounds__(kFixBlock, D == 3 ? 8 : 14)
 k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice<D>::Q> dst, Grid g, FixConst fc,
            Coll<double> k, Chunks ch, unsigned *__restrict__ flags)
 {
@@ -425,9 +456,8 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
 #pragma unroll
     for (int q = 0; q < Q; ++q) mx = max(mx, (unsigned)(w[q] >> 32) & 0x7fffffffu);
     const int eb = mx ? (int)(mx >> 20) : kFxMinExp;
-    bool ok = eb >= kFxMinExp && eb <= kFxMaxExp;
-    unsigned flag = 0u;
-    if (__all_sync(all, ok)) {
+    bool fine = __all_sync(all, eb >= kFxMinExp && eb <= kFxMaxExp);
+    if (fine) {
         long long X[Q], M = 0, J[3] = {0, 0, 0}, e1 = 0, e2 = 0;
 #pragma unroll
         for (int q = 0; q < Q; ++q) X[q] = fx_align((unsigned)(w[q] >> 32), (unsigned)w[q], eb);
@@ -446,23 +476,20 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
 #pragma unroll
         for (int a = 0; a < D; ++a) J[a] = fx_from_lane0(J[a]);
         FixCoef cf;
-        ok = fx_coefficients<D>(fx_from_lane0(M), J, fx_from_lane0(e1 + 2 * e2), fc, cf);
-        if (__all_sync(all, ok)) {
-            const FxSplit omc = fx_split(fc.omc), m = fx_split(M);
-            const int e0 = mx ? eb : 25;
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                long long t;
-                unsigned f;
-                fx_update(X[q], omc, fx_h<D>(cf, q), m, t, f);
-                w[q] = fx_to_double(t, f, e0);
-            }
-        } else {
-#pragma unroll
-            for (int q = 0; q < Q; ++q) w[q] = load(q);
-            flag = fx_collide_double<D>(w, k);
+        fine = __all_sync(all, fx_coefficients<D>(fx_from_lane0(M), J, fx_from_lane0(e1 + 2 * e2), fc, cf));
+        if (fine) {
+            const FxSplit m = fx_split(M);
+            const int shift = (eb - 1078) * (1 << 20);
+            fx_each_h<D>(cf, [&](int q, long long h) {
+                w[q] = (unsigned long long)__double_as_longlong(
+                    fx_to_double(fx_update(X[q], fc.omc, h, m), shift));
+            });
         }
-    } else {
+    }
+    unsigned flag = 0u;
+    if (!fine) {
+#pragma unroll
+        for (int q = 0; q < Q; ++q) w[q] = load(q);
         flag = fx_collide_double<D>(w, k);
     }
     if (active) {

@@ -38,6 +38,15 @@ template <int D> __host__ __device__ constexpr int cnorm2(int q)
 }
 template <int D> __host__ __device__ constexpr int opposite(int q) { return Lattice<D>::Q - 1 - q; }
 
+// Direction with lattice vector (x, y, z) (a vector of the lattice).
+template <int D> __host__ __device__ constexpr int direction_of(int x, int y, int z)
+{
+    const int r = x + 1 + 3 * (y + 1);      // place in the layer z
+    if (D == 2) return r;
+    if (z == 0) return r + 5;
+    return (r == 1 ? 0 : (r == 7 ? 4 : r - 2)) + (z > 0 ? 14 : 0);
+}
+
 // Per-site field of the magnetic-field term: one unit quaternion per site,
 // float4 for single-precision arithmetic, two double2 (DQuad) otherwise.
 struct __align__(16) DQuad {
