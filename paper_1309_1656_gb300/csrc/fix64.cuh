@@ -106,8 +106,29 @@ inline unsigned fx_bits(float v)
 
 #define FX_FN __host__ __device__ __forceinline__
 
+// sum X_q, sum i X_q and sum |i|^2 X_q.
+template <int D>
+FX_FN void fx_sums(const long long (&X)[Lattice<D>::Q], long long &M, long long (&J)[3], long long &E)
+{
+    constexpr int Q = Lattice<D>::Q;
+    long long e1 = 0, e2 = 0;
+    J[0] = J[1] = J[2] = 0;
+#pragma unroll
+    for (int q = 0; q < Q / 2; ++q) {
+        const long long s = X[q] + X[Q - 1 - q], d = X[Q - 1 - q] - X[q];
+        if (cnorm2<D>(q) == 1) e1 += s;
+        else e2 += s;
+        // direction Q - 1 - q is -q's: d carries the sign of its components
+        if (cx<D>(q)) J[0] += cx<D>(q) < 0 ? d : -d;
+        if (cy<D>(q)) J[1] += cy<D>(q) < 0 ? d : -d;
+        if (cz<D>(q)) J[2] += cz<D>(q) < 0 ? d : -d;
+    }
+    M = e1 + e2 + X[Q / 2];
+    E = e1 + 2 * e2;
+}
+
 // v = hi 2^32 + lo with lo signed: products of two splits then need signed
-// 32 x 32 -> 64-bit multiply-adds only.
+// 32 x 32 -> 64-bit multiply-adds only.  v < 2^63 - 2^31 (hi would wrap).
 struct FxSplit {
     int hi, lo;
 };
@@ -187,7 +208,7 @@ FX_FN long long fx_update(long long X, FxSplit omc, long long h, FxSplit m)
     return fx_mad(m.hi, g.hi, fx_mad(x.hi, omc.hi, cross >> 32));
 }
 
-// 1/x in q62 for nn = x 2^64, x in [1/2, 1): a single-precision reciprocal
+// 1/x in q61 for nn = x 2^64, x in [1/2, 1): a single-precision reciprocal
 // and two Newton steps r <- r + r (1 - x r) in integers, each product cut
 // below 2^-62.
 FX_FN long long fx_recip(unsigned long long nn)
@@ -202,8 +223,35 @@ FX_FN long long fx_recip(unsigned long long nn)
     const unsigned rh = (unsigned)((unsigned long long)r1 >> 32), rl = (unsigned)r1;
     const unsigned long long x1 = fx_umad(nh, rh, fx_umad(nh, rl, 0) >> 32) + (fx_umad(nl, rh, 0) >> 32);
     const int e1 = (int)(kFxOne - (long long)x1);       // < 2^20
-    const long long r = r1 + (fx_wide((int)(rh >> 1), e1) >> 29);
-    return r < 0 ? 0x7fffffffffffffffLL : r;            // x = 1/2
+    const long long r = r1 + (fx_wide((int)(rh >> 1), e1) >> 29);       // q62, up to 2^63
+    return (long long)((unsigned long long)r >> 1);
+}
+
+// J/n and E2/n - |j|^2 of a site.
+struct FixRatios {
+    FxSplit j[3];       // q64
+    long long jj;       // q64: |j|^2
+    long long ej;       // q60: E2/n - |j|^2
+};
+
+// From n, J, E2 (all in the same units); false outside the range of the form
+// (decided on high words): |j_a| < 3/8 (so |j|^2 < 1/2), 0 <= E2/n < 15/8.
+template <int D> FX_FN bool fx_ratios(long long n, const long long (&J)[3], long long E, FixRatios &o)
+{
+    const int nh = (int)(n >> 32), Eh = (int)(E >> 32), lim = (nh >> 2) + (nh >> 3);
+    auto mag = [](long long v) { return abs((int)(v >> 32)); };
+    bool ok = Eh >= 0 && (Eh >> 1) < nh - (nh >> 4) && mag(J[0]) < lim && mag(J[1]) < lim;
+    if (D == 3) ok = ok && mag(J[2]) < lim;
+    const int lz = fx_clz((unsigned)nh);    // 1..31 where ok
+    const FxSplit r = fx_split(fx_recip((unsigned long long)n << lz));
+    o.jj = 0;
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        o.j[a] = fx_split(fx_mul(fx_split(J[a] << lz), r) << 3);
+        o.jj += fx_mul(o.j[a], o.j[a]);
+    }
+    o.ej = 2 * fx_mul(fx_split((E >> 1) << (lz - 1)), r) - (o.jj >> 4);
+    return ok;
 }
 
 // h_i of all directions as ten basis values (q62).
@@ -214,44 +262,38 @@ struct FixCoef {
     long long qo[3];                // axis class: c4 j_a j_b, (a, b) = (0,1), (0,2), (1,2)
 };
 
-// From n, J, E2 (all in the same units); false outside the range of the form
-// (decided on high words).
-template <int D> FX_FN bool fx_coefficients(long long n, const long long (&J)[3], long long E, const FixConst &k,
-                                            FixCoef &c)
+// From j (q64), |j|^2 (q64) and d = E2/n - |j|^2 - d0 (q60); false where |d|
+// is not well below 1 or an |h_i| might reach 1 (the terms not looked at are bounded by
+// |j_a| < 3/8, see make_fix_const).
+template <int D>
+FX_FN bool fx_basis(const FxSplit (&j)[3], long long jj, long long d60, const FixConst &k, FixCoef &c)
 {
-    // |j_a| < 3/8 (so |j|^2 < 1/2), 0 <= E2/n < 2
-    const int nh = (int)(n >> 32), Eh = (int)(E >> 32), lim = (nh >> 2) + (nh >> 3);
     auto mag = [](long long v) { return abs((int)(v >> 32)); };
-    bool ok = Eh >= 0 && (Eh >> 1) < nh && mag(J[0]) < lim && mag(J[1]) < lim;
-    if (D == 3) ok = ok && mag(J[2]) < lim;
-    const int lz = fx_clz((unsigned)nh);    // 1..31 where ok
-    const FxSplit r = fx_split(fx_recip((unsigned long long)n << lz));
-    FxSplit j[3];       // q64
-    long long jj = 0;   // q64
 #pragma unroll
     for (int a = 0; a < D; ++a) {
-        j[a] = fx_split(fx_mul(fx_split(J[a] << lz), r) << 2);
         c.B[a] = fx_mul(k.c3, j[a]);
-        const long long sq = fx_mul(j[a], j[a]);
-        jj += sq;
-        c.qd[a] = fx_mul(k.c4, fx_split(sq));
+        c.qd[a] = fx_mul(k.c4, fx_split(fx_mul(j[a], j[a])));
     }
     c.qo[0] = fx_mul(k.c4, fx_split(fx_mul(j[0], j[1])));
     if (D == 3) {
         c.qo[1] = fx_mul(k.c4, fx_split(fx_mul(j[0], j[2])));
         c.qo[2] = fx_mul(k.c4, fx_split(fx_mul(j[1], j[2])));
     }
-    const long long d60 = fx_mul(fx_split((E >> 1) << (lz - 1)), r) - k.d0 - (jj >> 4);
-    ok = ok && mag(d60) < (1 << 28);
     const FxSplit d = fx_split(d60 << 3), s = fx_split(jj);     // q63, q64
     const long long g1 = fx_mul(k.ga[1], s);
     c.b0 = k.al[0] + fx_mul(k.ga[0], s) + 2 * fx_mul(k.be[0], d);
     c.b1 = k.al[1] + g1 + 2 * fx_mul(k.be[1], d);
     c.b2 = k.al[2] + (g1 >> (D == 3 ? 1 : 2)) + 2 * fx_mul(k.be[2], d);
-    // |h_i| < 1 for every direction: the other terms are bounded by |j_a| <
-    // 3/8 (make_fix_const)
     constexpr int q62 = 1 << 30;
-    return ok && mag(c.b0) < q62 && mag(c.b1) < q62 / 2 && mag(c.b2) < q62 / 4;
+    return mag(d60) < (1 << 28) - (1 << 20) && mag(c.b0) < q62 && mag(c.b1) < q62 / 2 && mag(c.b2) < q62 / 4;
+}
+
+template <int D> FX_FN bool fx_coefficients(long long n, const long long (&J)[3], long long E, const FixConst &k,
+                                            FixCoef &c)
+{
+    FixRatios r;
+    const bool ok = fx_ratios<D>(n, J, E, r);
+    return fx_basis<D>(r.j, r.jj, r.ej - k.d0, k, c) && ok;
 }
 
 // Calls f(q, h_q) for every direction, h_q in q62: the terms are shared
@@ -458,25 +500,15 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
     const int eb = mx ? (int)(mx >> 20) : kFxMinExp;
     bool fine = __all_sync(all, eb >= kFxMinExp && eb <= kFxMaxExp);
     if (fine) {
-        long long X[Q], M = 0, J[3] = {0, 0, 0}, e1 = 0, e2 = 0;
+        long long X[Q], M, J[3], E;
 #pragma unroll
         for (int q = 0; q < Q; ++q) X[q] = fx_align((unsigned)(w[q] >> 32), (unsigned)w[q], eb);
-#pragma unroll
-        for (int q = 0; q < Q / 2; ++q) {
-            const long long s = X[q] + X[Q - 1 - q], d = X[Q - 1 - q] - X[q];
-            if (cnorm2<D>(q) == 1) e1 += s;
-            else e2 += s;
-            // direction Q - 1 - q is -q's: d carries the sign of its components
-            if (cx<D>(q)) J[0] += cx<D>(q) < 0 ? d : -d;
-            if (cy<D>(q)) J[1] += cy<D>(q) < 0 ? d : -d;
-            if (cz<D>(q)) J[2] += cz<D>(q) < 0 ? d : -d;
-        }
-        M = e1 + e2 + X[Q / 2];
+        fx_sums<D>(X, M, J, E);
         // the coefficients from f's sums (formed by the site's four lanes alike)
 #pragma unroll
         for (int a = 0; a < D; ++a) J[a] = fx_from_lane0(J[a]);
         FixCoef cf;
-        fine = __all_sync(all, fx_coefficients<D>(fx_from_lane0(M), J, fx_from_lane0(e1 + 2 * e2), fc, cf));
+        fine = __all_sync(all, fx_coefficients<D>(fx_from_lane0(M), J, fx_from_lane0(E), fc, cf));
         if (fine) {
             const FxSplit m = fx_split(M);
             const int shift = (eb - 1078) * (1 << 20);

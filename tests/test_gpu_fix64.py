@@ -133,3 +133,30 @@ def test_two_buffer_step_is_the_same(q, d, dims):
         lat.rollout(5, 1)
         got = lat.get_state()
     assert np.array_equal(got, step(q, d, dims, 0.7, st, 5))
+
+
+@pytest.mark.parametrize("scale", [1.0, 0.25])
+@pytest.mark.parametrize("d,dims", [(2, (32, 4, 1)), (3, (16, 4, 2))])
+def test_density_near_a_power_of_two(q, d, dims, scale):
+    # 1/n at both ends of its normalised range: n = scale (1 +- 2^-k), k = 1..53
+    st = fields.random_populations(d, dims, seed=43)
+    b, N = st.shape[0], st.shape[2]
+    st *= 0.5 / st[:, 0].sum(0)
+    k = np.arange(N) % 54
+    n = np.where(np.arange(N) < N // 2, 1.0 + 2.0 ** -k.astype(float), 1.0 - 2.0 ** -(k + 1.0))
+    st[b // 2, 0] += n - st[:, 0].sum(0)
+    st *= scale
+    for steps in (1, 2):
+        got = step(q, d, dims, 0.8, st, steps)
+        assert worst(got, reference(q, d, dims, 0.8, st, steps)) < steps * TOL
+    with q.Lattice(d, dims, 0.8, 1.0, precision="fp64") as lat:
+        lat.set_state(st)
+        r, u, eps = lat.moments()
+        xi = lat.info()["xi"]
+    e = [(x, y, z) for z in ((-1, 0, 1) if d == 3 else (0,)) for y in (-1, 0, 1) for x in (-1, 0, 1)
+         if abs(x) + abs(y) + abs(z) < 3]
+    f = st[:, 0].astype(np.longdouble)
+    j = [sum(v[a] * f[i] for i, v in enumerate(e)) / f.sum(0) for a in range(d)]
+    E = sum(sum(map(abs, v)) * f[i] for i, v in enumerate(e)) / f.sum(0)
+    assert np.max(np.abs(u - xi * np.stack(j))) < TOL
+    assert np.max(np.abs(eps - 0.5 * xi * xi * (E - sum(a * a for a in j)))) < 4 * TOL
