@@ -186,17 +186,23 @@ __global__ void __launch_bounds__(kRedBlock)
 k_conserved_final(const double *__restrict__ partials, int nparts, double xi, int64_t N,
                   double *__restrict__ out)
 {
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int r = threadIdx.x; r < nparts; r += blockDim.x)
-#pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] += partials[(int64_t)r * 8 + i];
-    __shared__ double res[8];
-    block_sum_store<8>(acc, res);
+    // thread (r, i) sums component i of rows r, r + 32, ...: the double pipe
+    // (64 cycles per warp instruction) is what this block waits for, so no
+    // thread adds a component it does not keep (one thread per row with eight
+    // sums and shuffles over all of them: 7.4 us, this 2.5 us at 608 rows)
+    const int i = threadIdx.x & 7;
+    double acc = 0.0;
+    for (int r = threadIdx.x >> 3; r < nparts; r += kRedBlock / 8) acc += partials[(int64_t)r * 8 + i];
+    acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+    acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+    __shared__ double sh[kRedBlock / 32][8];
+    if ((threadIdx.x & 31) < 8) sh[threadIdx.x >> 5][i] = acc;
     __syncthreads();
     if (threadIdx.x < 8) {
-        const int i = threadIdx.x;
+        double t = 0.0;
+        for (int w = 0; w < kRedBlock / 32; ++w) t += sh[w][i];
         const double scale = i < 4 ? 1.0 : (i < 7 ? xi : 0.5 * xi * xi);
-        out[i] = res[i] * scale / (double)N;
+        out[i] = t * scale / (double)N;
     }
 }
 
@@ -302,7 +308,8 @@ int qlbm_create(qlbm_handle *out, int lattice, const int64_t dims[3], double tau
     if (e == cudaSuccess) e = cudaMalloc(&h->flags, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemsetAsync(h->flags, 0, sizeof(unsigned), h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    int64_t nred = (g.N + kRedBlock - 1) / kRedBlock;
+    // blocks of the reduction: at most one warp per 8-site chunk of a row
+    const int64_t nred = ((int64_t)((g.nx + 7) / 8) * g.ny * g.nz + kRedBlock / 32 - 1) / (kRedBlock / 32);
     h->nred = (int)(nred < 1024 ? nred : 1024);
     if (e == cudaSuccess) e = cudaMalloc(&h->partials, (size_t)h->nred * 8 * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->red_out, 8 * sizeof(double));

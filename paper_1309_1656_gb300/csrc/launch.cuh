@@ -8,7 +8,9 @@
 #include "internal.h"
 #include "adjoint.cuh"
 #include "fdkernels.cuh"
+#include "initeq.cuh"
 #include "kernels.cuh"
+#include "quadsum.cuh"
 #include "twopass.cuh"
 
 namespace qlbm {
@@ -70,7 +72,19 @@ inline InitConsts make_init(const qlbm_ctx *h)
     ic.eps0 = k.eps0;
     ic.beta0 = k.beta0;
     for (int i = 0; i < 3; ++i) ic.w[i] = k.w[i];
+    ic.rxi = 0x1p64 / k.xi;
+    ic.rK = 0x1p60 / k.K;
+    ic.umax = 0.375 * k.xi;
     return ic;
+}
+
+// The fixed-point coefficients of h_i = w_i P_i (omega = 1; independent of
+// beta0 and in range for both lattices).
+inline FixConst make_fix_unit(const qlbm_ctx *h)
+{
+    FixConst fc;
+    make_fix_const(h->hc, 1.0, &fc);
+    return fc;
 }
 
 template <class Codec> Codec make_codec(const qlbm_ctx *h);
@@ -121,7 +135,7 @@ template <int D, class Codec> struct Launchers {
     static cudaError_t init_eq(qlbm_ctx *h, const double *rho4, const double *u, const double *eps)
     {
         const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
-        k_init_eq<D, Codec><<<grd, blk, 0, h->stream>>>(planes(h), h->g, make_init(h),
+        k_init_eq<D, Codec><<<grd, blk, 0, h->stream>>>(planes(h), h->g, make_init(h), make_fix_unit(h),
                                                         make_codec<Codec>(h), rho4, u, eps);
         return cudaGetLastError();
     }
@@ -144,16 +158,54 @@ template <int D, class Codec> struct Launchers {
         return cudaGetLastError();
     }
 
+    // grid of the kernels with one warp per 8-site chunk
+    static dim3 quad_grid(const Chunks &ch) { return dim3((unsigned)((ch.total + kQuadBlock / 32 - 1) / (kQuadBlock / 32))); }
+
+    // codecs whose site sums are formed by one thread per site (4-byte values)
+    static constexpr bool kSiteSums = sizeof(typename QuadValue<Codec>::Raw) == 4;
+
     static cudaError_t moments(qlbm_ctx *h, double *rho4, double *u, double *eps)
     {
-        const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
+        const QuadRef ref = make_quad_ref(h->hc);
         const Planes<S, Q> pl = planes(h);
-        if (h->parity)
-            k_moments<D, Codec, true><<<grd, blk, 0, h->stream>>>(pl, h->g, make_codec<Codec>(h),
-                                                                  h->hc.xi, rho4, u, eps);
-        else
-            k_moments<D, Codec, false><<<grd, blk, 0, h->stream>>>(pl, h->g, make_codec<Codec>(h),
-                                                                   h->hc.xi, rho4, u, eps);
+        const Codec codec = make_codec<Codec>(h);
+        const double xi = h->hc.xi, e = 0.5 * xi * xi;
+        const MomentScale sc{xi * 0x1p-62, e * 0x1p-62, xi, e};
+        if constexpr (kSiteSums) {
+            const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
+            if (h->parity)
+                k_moments_site<D, Codec, true><<<grd, blk, 0, h->stream>>>(pl, h->g, codec, ref, sc, rho4, u, eps);
+            else
+                k_moments_site<D, Codec, false><<<grd, blk, 0, h->stream>>>(pl, h->g, codec, ref, sc, rho4, u, eps);
+        } else {
+            const Chunks ch = make_chunks(h->g);
+            if (h->parity)
+                k_moments<D, Codec, true><<<quad_grid(ch), kQuadBlock, 0, h->stream>>>(pl, h->g, codec, ch, ref, sc,
+                                                                                       rho4, u, eps);
+            else
+                k_moments<D, Codec, false><<<quad_grid(ch), kQuadBlock, 0, h->stream>>>(pl, h->g, codec, ch, ref, sc,
+                                                                                        rho4, u, eps);
+        }
+        return cudaGetLastError();
+    }
+
+    // Launches conserved_partial's kernel for a buffer parity (grid > 0), or
+    // reports its resident blocks per SM (grid 0).
+    template <bool SWAPPED> static cudaError_t conserved_launch(qlbm_ctx *h, int grid, int *resident)
+    {
+        if constexpr (kSiteSums) {
+            if (!grid)
+                return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                    resident, k_conserved_partial_df<D, Codec, SWAPPED>, kRedBlock, 0);
+            k_conserved_partial_df<D, Codec, SWAPPED><<<grid, kRedBlock, 0, h->stream>>>(
+                planes(h), h->g, make_codec<Codec>(h), h->partials);
+        } else {
+            if (!grid)
+                return cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, k_conserved_partial<D, Codec, SWAPPED>,
+                                                                     kRedBlock, 0);
+            k_conserved_partial<D, Codec, SWAPPED><<<grid, kRedBlock, 0, h->stream>>>(
+                planes(h), h->g, make_codec<Codec>(h), make_chunks(h->g), make_quad_ref(h->hc), h->partials);
+        }
         return cudaGetLastError();
     }
 
@@ -163,22 +215,14 @@ template <int D, class Codec> struct Launchers {
             // one whole wave of resident blocks (a fixed count left a
             // partial second wave); found once per handle
             int a = 0, b = 0;
-            cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, k_conserved_partial<D, Codec, false>,
-                                                                          kRedBlock, 0);
-            if (e == cudaSuccess)
-                e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_conserved_partial<D, Codec, true>, kRedBlock, 0);
+            cudaError_t e = conserved_launch<false>(h, 0, &a);
+            if (e == cudaSuccess) e = conserved_launch<true>(h, 0, &b);
             if (e != cudaSuccess) return e;
             const int64_t wave = (int64_t)(a < b ? a : b) * h->sms;
             h->red_grid = (int)(wave >= 1 && wave < h->nred ? wave : h->nred);
         }
-        const Planes<S, Q> pl = planes(h);
-        if (h->parity)
-            k_conserved_partial<D, Codec, true><<<h->red_grid, kRedBlock, 0, h->stream>>>(
-                pl, h->g, make_codec<Codec>(h), h->partials);
-        else
-            k_conserved_partial<D, Codec, false><<<h->red_grid, kRedBlock, 0, h->stream>>>(
-                pl, h->g, make_codec<Codec>(h), h->partials);
-        return cudaGetLastError();
+        return h->parity ? conserved_launch<true>(h, h->red_grid, nullptr)
+                         : conserved_launch<false>(h, h->red_grid, nullptr);
     }
 
     static cudaError_t adjoint(qlbm_ctx *h, const void *state, const void *lam_in, void *lam_out)
@@ -281,13 +325,15 @@ template <int D, class Codec> struct Launchers {
 
     static cudaError_t negative_eq(qlbm_ctx *h, unsigned long long *count, unsigned *mask)
     {
-        const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
+        const Chunks ch = make_chunks(h->g);
+        const QuadRef ref = make_quad_ref(h->hc);
+        const Codec codec = make_codec<Codec>(h);
         if (h->parity)
-            k_negative_eq<D, Codec, true><<<grd, blk, 0, h->stream>>>(planes(h), h->g, make_codec<Codec>(h),
-                                                                      make_init(h), count, mask);
+            k_negative_eq<D, Codec, true><<<quad_grid(ch), kQuadBlock, 0, h->stream>>>(
+                planes(h), h->g, codec, ch, ref, make_fix_unit(h), make_init(h), count, mask);
         else
-            k_negative_eq<D, Codec, false><<<grd, blk, 0, h->stream>>>(planes(h), h->g, make_codec<Codec>(h),
-                                                                       make_init(h), count, mask);
+            k_negative_eq<D, Codec, false><<<quad_grid(ch), kQuadBlock, 0, h->stream>>>(
+                planes(h), h->g, codec, ch, ref, make_fix_unit(h), make_init(h), count, mask);
         return cudaGetLastError();
     }
 
