@@ -339,6 +339,7 @@ void qlbm_destroy(qlbm_handle h)
     if (h->dtau_acc) cudaFree(h->dtau_acc);
     if (h->scratch_state) cudaFree(h->scratch_state);
     if (h->fd_fail) cudaFree(h->fd_fail);
+    if (h->fd_rho) cudaFree(h->fd_rho);
     if (h->qfield) cudaFree(h->qfield);
     if (h->neg_count) cudaFree(h->neg_count);
     if (h->graph) cudaGraphExecDestroy(h->graph);

@@ -321,11 +321,17 @@ template <int D> __device__ __forceinline__ Fd3f fd3f(float x)
     return r;
 }
 
+// What a Newton step needs of the Jacobian: 1/g_s, c_s / g_s and the inverse
+// of the Schur complement.
+struct FdJacF {
+    float ig1, ig2, cg1, cg2, rden;
+};
+
 // The Newton iteration of fd_params_site in single precision, from the
 // classical start: true and (t = log beta, nu_up, nu_dn) to ~1e-6 when it
-// settles within 20 iterations.
+// settles within 20 iterations; J: the last step's Jacobian.
 template <int D>
-__device__ bool fd_newton_f(float nup, float ndn, float n, float eps, float &t, float &nu1, float &nu2)
+__device__ bool fd_newton_f(float nup, float ndn, float n, float eps, float &t, float &nu1, float &nu2, FdJacF &J)
 {
     constexpr float h = 0.5f * D;
     constexpr float hl2pi = h * 1.83787707f;   // h log 2 pi
@@ -345,6 +351,7 @@ __device__ bool fd_newton_f(float nup, float ndn, float n, float eps, float &t, 
         const float den = -(h + 1.f) + h * (c1 * ig1 + c2 * ig2);
         float dt = (c1 * ig1 * r1 + c2 * ig2 * r2 - r3) / den;
         if (!(dt == dt)) return false;
+        J = FdJacF{ig1, ig2, c1 * ig1, c2 * ig2, 1.f / den};
         dt = fmaxf(-1.f, fminf(1.f, dt));
         const float d1 = fmaxf(-10.f, fminf(10.f, (h * dt - r1) * ig1));
         const float d2 = fmaxf(-10.f, fminf(10.f, (h * dt - r2) * ig2));
@@ -427,6 +434,98 @@ __device__ FdParams fd_params_nested(double n, double Sx, double Sy, double Sz, 
     return p;
 }
 
+// 1/x for x within single precision's range: the float reciprocal and two
+// Newton steps.
+__device__ __forceinline__ double fd_recip(double x)
+{
+    double r = (double)(1.0f / (float)x);
+    r = fma(r, fma(-x, r, 1.0), r);
+    return fma(r, fma(-x, r, 1.0), r);
+}
+
+// F_{h-2}, F_{h-1}, F_h at a single-precision x in [-8, 1) from the
+// polynomials on intervals of 1/4; F_{h-3} in single precision.
+template <int D> __device__ __forceinline__ Fd3 fd3_poly(float x, float &hm3)
+{
+    const int i = (int)((x - (float)FD_PX0) * 4.f);
+    const float c = (float)FD_PX0 + 0.125f + 0.25f * (float)i, tf = x - c;
+    const double t = (double)x - (double)c;     // (tf is rounded where |x| is small)
+    const double(*p)[3] = FD_POLY[D - 2][i];
+    Fd3 r{p[FD_PDEG][0], p[FD_PDEG][1], p[FD_PDEG][2]};
+#pragma unroll
+    for (int j = FD_PDEG - 1; j >= 0; --j) {
+        r.m2 = fma(r.m2, t, p[j][0]);
+        r.m1 = fma(r.m1, t, p[j][1]);
+        r.h = fma(r.h, t, p[j][2]);
+    }
+    const float(*pf)[1] = FDF_POLY[D - 2][i];
+    hm3 = pf[FD_PDEGF][0];
+#pragma unroll
+    for (int j = FD_PDEGF - 1; j >= 0; --j) hm3 = fmaf(hm3, tf, pf[j][0]);
+    return r;
+}
+
+// One pass in double from the single-precision solution (b0 = e^t, nu1, nu2;
+// J its Jacobian, good to ~1e-5): F is evaluated in double once, at that
+// point x_0.  The residuals' relative form rho_s = F_{h-1}(nu_s) A/n_s - 1,
+// rho_3 = h A/beta sum F_h/(n eps) - 1 gives a correction delta_0 ~ 1e-6 with
+// an error ~1e-11; the residuals at x_0 + delta_0 come from the Taylor series
+// (F_k' = F_{k-1}; terms beyond delta^2 are below delta^3 / 6 < 2e-17), and
+// their correction brings the error to ~1e-16.  So the solve takes ~170
+// double-precision instructions instead of three evaluations of series of up
+// to 40 terms.  False (nothing written) where the point leaves the tables'
+// range or the first correction is not small.
+template <int D>
+__device__ __forceinline__ bool fd_one_pass(double nup, double ndn, double neps, float b0f, float nu1f, float nu2f,
+                                            const FdJacF &J, FdParams &p)
+{
+    constexpr float hf = 0.5f * D;
+    constexpr double h = 0.5 * D;
+    if (!(nu1f >= (float)FD_PX0 && nu1f < 1.f && nu2f >= (float)FD_PX0 && nu2f < 1.f)) return false;
+    // within single precision's range (the reciprocals)
+    if (!(b0f > 1e-12f && b0f < 1e12f && nup < 1e12 && ndn > 1e-12 && neps > 1e-12 && neps < 1e12)) return false;
+    const double b0 = b0f, rb = fd_recip(b0), q = kTwoPi * rb;
+    double A = q;           // (2 pi / b0)^h
+    if (D == 3) {           // q sqrt(q): the float square root and two Newton steps
+        const float sf = sqrtf((float)q);
+        const double hs = (double)(0.5f / sf);
+        double s = sf;
+        s = fma(fma(-s, s, q), hs, s);
+        s = fma(fma(-s, s, q), hs, s);
+        A = q * s;
+    }
+    float G1, G2;           // F_{h-3}
+    const Fd3 F1 = fd3_poly<D>(nu1f, G1), F2 = fd3_poly<D>(nu2f, G2);
+    const double a1 = A * fd_recip(nup), a2 = A * fd_recip(ndn), a3 = h * A * rb * fd_recip(neps);
+    auto solve = [&](float r1, float r2, float r3, float &dt, float &d1, float &d2) {
+        dt = (J.cg1 * r1 + J.cg2 * r2 - r3) * J.rden;
+        d1 = (hf * dt - r1) * J.ig1;
+        d2 = (hf * dt - r2) * J.ig2;
+    };
+    float t0, x1, x2, t1, y1, y2;
+    solve((float)fma(F1.m1, a1, -1.0), (float)fma(F2.m1, a2, -1.0), (float)fma(F1.h + F2.h, a3, -1.0), t0, x1, x2);
+    if (!(fmaxf(fabsf(t0), fmaxf(fabsf(x1), fabsf(x2))) <= 5e-6f)) return false;
+    // at x_0 + delta_0
+    const double dt = t0, dx1 = x1, dx2 = x2;
+    const double m1 = fma(dx1, fma(dx1, (double)(0.5f * G1), F1.m2), F1.m1);
+    const double m2 = fma(dx2, fma(dx2, (double)(0.5f * G2), F2.m2), F2.m1);
+    const double hh = fma(dx1, fma(0.5 * dx1, F1.m2, F1.m1), F1.h) + fma(dx2, fma(0.5 * dx2, F2.m2, F2.m1), F2.h);
+    const double z = h * dt, E = fma(z, fma(z, 0.5, -1.0), 1.0);        // e^(-h dt)
+    const double B = fma(dt, fma(dt, 0.5, -1.0), 1.0);                  // e^(-dt)
+    solve((float)fma(m1 * E, a1, -1.0), (float)fma(m2 * E, a2, -1.0), (float)fma(hh * E, a3 * B, -1.0), t1, y1, y2);
+    const double et = dt + (double)t1;
+    p.beta = fma(b0, fma(et * et, 0.5, et), b0);
+    const double rbeta = rb * fma(et, fma(et, 0.5, -1.0), 1.0);
+    p.mu_up = ((double)nu1f + (dx1 + (double)y1)) * rbeta;
+    p.mu_dn = ((double)nu2f + (dx2 + (double)y2)) * rbeta;
+    // (2 pi/beta)^h F_{h-1} at the solution
+    const double AE = A * fma(-h, (double)t1, 1.0) * E;
+    p.n_up = AE * fma((double)y1, F1.m2, m1);
+    p.n_dn = AE * fma((double)y2, F2.m2, m2);
+    p.status = 0;
+    return true;
+}
+
 // Newton's method on
 //   r_1 = log F_{h-1}(nu_up) - h t + h log 2 pi - log n_up
 //   r_2 = log F_{h-1}(nu_dn) - h t + h log 2 pi - log n_dn
@@ -460,13 +559,17 @@ __device__ FdParams fd_params_site(double n, double Sx, double Sy, double Sz, do
         return p;
     }
     const bool split = nS > 0.0;
+    // the single-precision solution, and one pass in double from it
+    float tf = 0.f, n1f = 0.f, n2f = 0.f;
+    FdJacF J;
+    const bool start = fd_newton_f<D>((float)nup, (float)ndn, (float)n, (float)eps, tf, n1f, n2f, J);
+    if (start && fd_one_pass<D>(nup, ndn, n * eps, expf(tf), n1f, split ? n2f : n1f, J, p)) return p;
     const double lA = log(nup), lB = split ? log(ndn) : lA, lC = log(n * eps / h);
     double t = log(h / eps);
     double nu1 = lA - hl2pi + h * t, nu2 = lB - hl2pi + h * t;
     // start from the single-precision solution (~1e-6) where it settles: two
     // double iterations then reach rounding level instead of four
-    float tf, n1f, n2f;
-    if (fd_newton_f<D>((float)nup, (float)ndn, (float)n, (float)eps, tf, n1f, n2f)) {
+    if (start) {
         t = tf;
         nu1 = n1f;
         nu2 = split ? (double)n2f : nu1;
@@ -527,7 +630,8 @@ __device__ FdParamsF fd_params_site_f(float n, float Sx, float Sy, float Sz, flo
     FdParamsF p;
     const float nS = sqrtf(Sx * Sx + Sy * Sy + Sz * Sz);
     float t, nu1, nu2;
-    if (!fd_newton_f<D>(0.5f * (n + nS), 0.5f * (n - nS), n, eps, t, nu1, nu2)) {
+    FdJacF J;
+    if (!fd_newton_f<D>(0.5f * (n + nS), 0.5f * (n - nS), n, eps, t, nu1, nu2, J)) {
         // invalid or unsettled: the double solve decides
         const FdParams q = fd_params_site<D>(n, Sx, Sy, Sz, eps);
         p.beta = (float)q.beta;

@@ -420,8 +420,11 @@ __device__ __forceinline__ long long fx_from_lane0(long long v)
 
 // The step of one component in double (collide's formulas), for warps with a
 // site outside the fixed-point form; lane c = 0 holds f, 1..3 the spins.
-template <int D>
-__device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[Lattice<D>::Q], const Coll<double> &k)
+// FD: the equilibrium is built from the component R of a rebuilt density
+// matrix instead of M (the flag then looks at n only).
+template <int D, bool FD>
+__device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[Lattice<D>::Q], const Coll<double> &k,
+                                                      double R)
 {
     constexpr int Q = Lattice<D>::Q;
     double M = 0.0, J[3] = {0.0, 0.0, 0.0}, E = 0.0;
@@ -448,25 +451,27 @@ __device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[La
         const double v = __longlong_as_double((long long)w[q]);
         const double t = cx<D>(q) * jx + cy<D>(q) * jy + cz<D>(q) * jz;
         const double h = k.w[cnorm2<D>(q)] * fma(t, fma(k.c4, t, k.c3), bq[cnorm2<D>(q)]);
-        w[q] = (unsigned long long)__double_as_longlong(fma(k.omega, fma(h, M, -v), v));
+        w[q] = (unsigned long long)__double_as_longlong(fma(k.omega, fma(h, FD ? R : M, -v), v));
     }
     double sum = (threadIdx.x & 3) ? fabs(M) : fabs(be);
     sum += __shfl_xor_sync(all, sum, 1, 4);
     sum += __shfl_xor_sync(all, sum, 2, 4);
     unsigned flag = 0u;
     if (!(n > 0.0)) flag |= n == n ? FLAG_NONPOSITIVE : FLAG_NONFINITE;
-    if (!(sum < 1e30)) flag |= FLAG_NONFINITE;
+    if (!FD && !(sum < 1e30)) flag |= FLAG_NONFINITE;
     return flag;
 }
 
 // One step of FP64 storage: an even or odd AA step in place (addressing as
 // k_step_aa; src and dst the same planes) or the two-buffer step of the
 // reverse mode (as k_step_push), with the same arithmetic in all three.
+// With FD the equilibrium is built from a density matrix per site (rho, Eq.
+// WeqDiscr) instead of the populations' own; P_i keeps their u and eps.
 enum : int { FIX_EVEN = 0, FIX_ODD = 1, FIX_PUSH = 2 };
-template <int D, int MODE>
+template <int D, int MODE, bool FD>
 __global__ void __launch_bounds__(kFixBlock, D == 3 ? 8 : 14)
 k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice<D>::Q> dst, Grid g, FixConst fc,
-           Coll<double> k, Chunks ch, unsigned *__restrict__ flags)
+           Coll<double> k, Chunks ch, const DQuad *__restrict__ rho, unsigned *__restrict__ flags)
 {
     constexpr int Q = Lattice<D>::Q;
     const unsigned all = 0xffffffffu;
@@ -498,6 +503,8 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
 #pragma unroll
     for (int q = 0; q < Q; ++q) mx = max(mx, (unsigned)(w[q] >> 32) & 0x7fffffffu);
     const int eb = mx ? (int)(mx >> 20) : kFxMinExp;
+    double R = 0.0;
+    if (FD) R = reinterpret_cast<const double *>(rho + si.s)[c];
     bool fine = __all_sync(all, eb >= kFxMinExp && eb <= kFxMaxExp);
     if (fine) {
         long long X[Q], M, J[3], E;
@@ -510,6 +517,12 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
         FixCoef cf;
         fine = __all_sync(all, fx_coefficients<D>(fx_from_lane0(M), J, fx_from_lane0(E), fc, cf));
         if (fine) {
+            if (FD) {       // rho's component in the units of M
+                const int rh = __double2hiint(R), e = (rh >> 20) & 0x7ff;
+                const bool zero = e <= eb - 70;     // below U / 2^13
+                fine = __all_sync(all, zero || (e < eb + 5 && mx != 0u));
+                M = zero ? 0 : __double2ll_rn(__hiloint2double(rh + (1080 - eb) * (1 << 20), __double2loint(R)));
+            }
             const FxSplit m = fx_split(M);
             const int shift = (eb - 1078) * (1 << 20);
             fx_each_h<D>(cf, [&](int q, long long h) {
@@ -522,7 +535,7 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
     if (!fine) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) w[q] = load(q);
-        flag = fx_collide_double<D>(w, k);
+        flag = fx_collide_double<D, FD>(w, k, R);
     }
     if (active) {
         const int so = si.s + g.zero;   // store addresses formed anew (see k_step_aa)

@@ -7,6 +7,11 @@ precision on the GPU, for k = -1/2, 1/2, 3/2 (D3Q19) and k = 1 (D2Q9).
   1 <= x < 49  Chebyshev series on 24 intervals of width 2        (CHEB)
   x >= 49      x^(k+1)/Gamma(k+2) sum_n 2 eta(2n) (k+1)k...(k+2-2n) x^-2n  (ASYM)
 
+For -8 <= x < 1, where one evaluation serves the one-pass solve, POLY holds
+polynomials in x - c on 36 intervals of width 1/4 (c the centre) for
+(F_{h-2}, F_{h-1}, F_h), h = 1 and 3/2, interpolated at the Chebyshev points
+(error below 1e-18 of F_k), and POLYF those of F_{h-3} in single precision.
+
 Values come from mpmath at 40 digits (polylog and altzeta); the FDF_*
 tables are single-precision truncations of the same expansions.  Run with
 `python gen_fd_tables.py` from this directory; the output is committed so
@@ -21,6 +26,7 @@ mp.mp.dps = 40
 KS = [mp.mpf(-1) / 2, mp.mpf(1) / 2, mp.mpf(3) / 2, mp.mpf(1)]
 NSER, NTAY, NINT, WIDTH, X0, NCHEB, NASYM = 40, 34, 24, 2, 1, 24, 9
 NSERF, NTAYF, NCHEBF, NASYMF = 20, 17, 10, 4
+PX0, PINT, PDEG, PDEGF = -8, 36, 10, 4
 
 
 def F(k, x):
@@ -37,6 +43,19 @@ def cheb_coeffs(k, a, b, n):
         c.append(2 * s / n)
     c[0] /= 2
     return c
+
+
+def poly_coeffs(k, c, r, deg):
+    """Monomial coefficients in x - c of the interpolant of F_k of degree deg
+    at the Chebyshev points of [c - r, c + r]."""
+    n = deg + 1
+    t = [r * mp.cos(mp.pi * (m + mp.mpf(1) / 2) / n) for m in range(n)]
+    A = mp.matrix(n, n)
+    for i in range(n):
+        for j in range(n):
+            A[i, j] = (t[i] / r) ** j
+    v = mp.lu_solve(A, mp.matrix([F(k, c + x) for x in t]))
+    return [v[j] / r ** j for j in range(n)]
 
 
 def fmt(v):
@@ -109,6 +128,19 @@ def main():
     out.append("__constant__ float FDF_ASYM[3][FDF_NASYM] = {")
     out += ["  {" + ", ".join(fmtf(v) for v in row[:NASYMF]) + "}," for row in asym]
     out.append("};")
+    # polynomials on the intervals of the one-pass solve
+    out.append("#define FD_PX0 %d\n#define FD_PINT %d\n#define FD_PDEG %d\n#define FD_PDEGF %d" % (PX0, PINT, PDEG, PDEGF))
+    for name, typ, deg, cols, f in (("FD_POLY", "double", PDEG, 3, fmt), ("FDF_POLY", "float", PDEGF, 1, fmtf)):
+        out.append("static __device__ const %s %s[2][FD_PINT][%s + 1][%d] = {" % (typ, name, "FD_PDEG" if cols == 3 else "FD_PDEGF", cols))
+        for h in (mp.mpf(1), mp.mpf(3) / 2):
+            out.append("  {")
+            for i in range(PINT):
+                c = mp.mpf(PX0) + (i + mp.mpf(1) / 2) / 4
+                ks = [h - 2, h - 1, h] if cols == 3 else [h - 3]
+                p = [poly_coeffs(k, c, mp.mpf(1) / 8, deg) for k in ks]
+                out.append("    {" + ", ".join("{" + ", ".join(f(q[j]) for q in p) + "}" for j in range(deg + 1)) + "},")
+            out.append("  },")
+        out.append("};")
     here = os.path.dirname(os.path.abspath(__file__))
     with open(os.path.join(here, "fd_tables.h"), "w") as f:
         f.write("\n".join(out) + "\n")

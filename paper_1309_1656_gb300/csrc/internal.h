@@ -68,6 +68,7 @@ struct qlbm_ctx {
     void *qfield = nullptr;             // per-site field: N unit quaternions (float4, or DQuad for FP64)
     double rot[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};   // its per-step spin rotation
     unsigned long long *fd_fail = nullptr;   // device counter of unresolved sites
+    void *fd_rho = nullptr;             // density matrices of the step through the parameters (DQuad per site)
     unsigned long long *neg_count = nullptr; // device counter of the negative-equilibrium diagnostic
     size_t state_bytes() const { return (size_t)b * 4 * (size_t)g.P * elem_bytes; }
     size_t lam_bytes() const { return (size_t)b * 4 * (size_t)g.P * (prec == QLBM_FP64 ? 8 : 4); }
@@ -117,9 +118,11 @@ const LatticeOps *ops_d3q19_fp64df();
 // the double-float step on FP64 storage (kernels_<lattice>_fp64df.cu)
 template <int D> cudaError_t step_f64df(qlbm_ctx *h, bool odd);
 // The FP64 step on the integer pipes (kernels_<lattice>_fp64_fix.cu): mode 0
-// even AA step, 1 odd, 2 two-buffer step from src to dst.  False, with nothing
-// launched, where it does not apply (a magnetic field; omega > 2).
-template <int D> bool step_fix(qlbm_ctx *h, int mode, const void *src, void *dst, cudaError_t *err);
+// even AA step, 1 odd, 2 two-buffer step from src to dst; rho: the density
+// matrices (DQuad per site) the equilibrium is built from, or NULL for the
+// populations' own.  False, with nothing launched, where it does not apply (a
+// magnetic field; omega > 2).
+template <int D> bool step_fix(qlbm_ctx *h, int mode, const void *src, void *dst, const void *rho, cudaError_t *err);
 
 inline const LatticeOps *lattice_ops(int d, int prec)
 {

@@ -6,7 +6,7 @@
 
 namespace qlbm {
 
-template <int D> bool step_fix(qlbm_ctx *h, int mode, const void *src, void *dst, cudaError_t *err)
+template <int D> bool step_fix(qlbm_ctx *h, int mode, const void *src, void *dst, const void *rho, cudaError_t *err)
 {
     FixConst fc;
     if (h->mag != FIELD_NONE || !make_fix_const(h->hc, h->dt / h->tau, &fc)) return false;
@@ -15,14 +15,14 @@ template <int D> bool step_fix(qlbm_ctx *h, int mode, const void *src, void *dst
     const Planes<double, Lattice<D>::Q> s = L::template planes_of<double>(h, src), d = L::template planes_of<double>(h, dst);
     const Coll<double> k = make_coll<double>(h);
     const dim3 blk(kFixBlock), grd((unsigned)((ch.total + kFixBlock / 32 - 1) / (kFixBlock / 32)));
-    switch (mode) {
-    case FIX_EVEN: k_step_fix<D, FIX_EVEN><<<grd, blk, 0, h->stream>>>(s, d, h->g, fc, k, ch, h->flags); break;
-    case FIX_ODD: k_step_fix<D, FIX_ODD><<<grd, blk, 0, h->stream>>>(s, d, h->g, fc, k, ch, h->flags); break;
-    default: k_step_fix<D, FIX_PUSH><<<grd, blk, 0, h->stream>>>(s, d, h->g, fc, k, ch, h->flags); break;
-    }
+    const DQuad *r = static_cast<const DQuad *>(rho);
+    auto launch = [&](auto kernel) { kernel<<<grd, blk, 0, h->stream>>>(s, d, h->g, fc, k, ch, r, h->flags); };
+    if (mode == FIX_PUSH) launch(k_step_fix<D, FIX_PUSH, false>);
+    else if (mode == FIX_ODD) launch(rho ? k_step_fix<D, FIX_ODD, true> : k_step_fix<D, FIX_ODD, false>);
+    else launch(rho ? k_step_fix<D, FIX_EVEN, true> : k_step_fix<D, FIX_EVEN, false>);
     *err = cudaGetLastError();
     return true;
 }
-template bool step_fix<3>(qlbm_ctx *, int, const void *, void *, cudaError_t *);
+template bool step_fix<3>(qlbm_ctx *, int, const void *, void *, const void *, cudaError_t *);
 
 }  // namespace qlbm

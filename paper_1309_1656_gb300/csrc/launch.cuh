@@ -169,8 +169,7 @@ template <int D, class Codec> struct Launchers {
         const QuadRef ref = make_quad_ref(h->hc);
         const Planes<S, Q> pl = planes(h);
         const Codec codec = make_codec<Codec>(h);
-        const double xi = h->hc.xi, e = 0.5 * xi * xi;
-        const MomentScale sc{xi * 0x1p-62, e * 0x1p-62, xi, e};
+        const MomentScale sc = moment_scale(h);
         if constexpr (kSiteSums) {
             const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
             if (h->parity)
@@ -242,7 +241,7 @@ template <int D, class Codec> struct Launchers {
         if constexpr (std::is_same<Codec, CodecF64>::value) {
             // the arithmetic of the step it stands for, bit for bit
             cudaError_t e;
-            if (step_fix<D>(h, 2, src, dst, &e)) return e;
+            if (step_fix<D>(h, 2, src, dst, nullptr, &e)) return e;
         }
         const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
         return with_field(h->mag, [&](auto fc) {
@@ -287,17 +286,38 @@ template <int D, class Codec> struct Launchers {
         return cudaGetLastError();
     }
 
+    static MomentScale moment_scale(const qlbm_ctx *h)
+    {
+        const double xi = h->hc.xi, e = 0.5 * xi * xi;
+        return MomentScale{xi * 0x1p-62, e * 0x1p-62, xi, e};
+    }
+
+    static cudaError_t fd_launch(qlbm_ctx *h, const FdOut &o)
+    {
+        const QuadRef ref = make_quad_ref(h->hc);
+        const MomentScale sc = moment_scale(h);
+        const Codec codec = make_codec<Codec>(h);
+        const Planes<S, Q> pl = planes(h);
+        if constexpr (kSiteSums) {
+            const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
+            if (h->parity)
+                k_fd_params_site<D, Codec, true><<<grd, blk, 0, h->stream>>>(pl, h->g, codec, ref, sc, o);
+            else
+                k_fd_params_site<D, Codec, false><<<grd, blk, 0, h->stream>>>(pl, h->g, codec, ref, sc, o);
+        } else {
+            const Chunks ch = make_chunks(h->g);
+            const dim3 grd((unsigned)((ch.total + kFdBlock / 8 - 1) / (kFdBlock / 8)));     // 4 chunks per warp
+            if (h->parity)
+                k_fd_params<D, Codec, true><<<grd, kFdBlock, 0, h->stream>>>(pl, h->g, codec, ch, ref, sc, o);
+            else
+                k_fd_params<D, Codec, false><<<grd, kFdBlock, 0, h->stream>>>(pl, h->g, codec, ch, ref, sc, o);
+        }
+        return cudaGetLastError();
+    }
+
     static cudaError_t fd_params(qlbm_ctx *h, double *beta, double *mu_up, double *mu_dn, double *axis)
     {
-        const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
-        const FdArgs a{h->hc.beta0, h->hc.xi};
-        if (h->parity)
-            k_fd_params<D, Codec, true><<<grd, blk, 0, h->stream>>>(planes(h), h->g, make_codec<Codec>(h), a, beta,
-                                                                    mu_up, mu_dn, axis, h->fd_fail);
-        else
-            k_fd_params<D, Codec, false><<<grd, blk, 0, h->stream>>>(planes(h), h->g, make_codec<Codec>(h), a, beta,
-                                                                     mu_up, mu_dn, axis, h->fd_fail);
-        return cudaGetLastError();
+        return fd_launch(h, FdOut{beta, mu_up, mu_dn, axis, nullptr, h->fd_fail, h->flags});
     }
 
     static cudaError_t fd_params_adjoint(qlbm_ctx *h, const double *gbeta, const double *gmu_up,

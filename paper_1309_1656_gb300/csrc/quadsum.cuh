@@ -294,6 +294,28 @@ struct MomentScale {
     double u62, e62, u, e;
 };
 
+// n and S (s.dM), u and eps of a site from its sums.
+template <int D>
+__device__ __forceinline__ void site_finish(SiteSums &s, const MomentScale &sc, double (&uu)[3], double &eps)
+{
+    FixRatios r;
+    if (s.fine && fx_ratios<D>(s.M[0], s.J, s.E, r)) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s.dM[c] = quad_double(s.M[c], s.unit[c]);
+#pragma unroll
+        for (int a = 0; a < D; ++a) uu[a] = (double)((((long long)r.j[a].hi << 32) + r.j[a].lo) >> 2) * sc.u62;
+        eps = (double)(r.ej << 2) * sc.e62;
+        return;
+    }
+    site_to_double(s);
+    const double rn = 1.0 / s.dM[0];
+    const double jx = s.dJ[0] * rn, jy = s.dJ[1] * rn, jz = D == 3 ? s.dJ[2] * rn : 0.0;
+    uu[0] = sc.u * jx;
+    uu[1] = sc.u * jy;
+    uu[2] = sc.u * jz;
+    eps = sc.e * (s.dE * rn - (jx * jx + jy * jy + jz * jz));
+}
+
 template <int D, class Codec, bool SWAPPED>
 __global__ void __launch_bounds__(kStepBlock, 4)
 k_moments_site(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Codec codec, QuadRef ref, MomentScale sc,
@@ -303,23 +325,8 @@ k_moments_site(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Codec 
     if (!site_of_block(g, si)) return;
     SiteSums s;
     site_sums<D, Codec, SWAPPED>(pl, g, si, codec, ref, s);
-    FixRatios r;
     double uu[3], ee;
-    if (s.fine && fx_ratios<D>(s.M[0], s.J, s.E, r)) {
-#pragma unroll
-        for (int c = 0; c < 4; ++c) s.dM[c] = quad_double(s.M[c], s.unit[c]);
-#pragma unroll
-        for (int a = 0; a < D; ++a) uu[a] = (double)((((long long)r.j[a].hi << 32) + r.j[a].lo) >> 2) * sc.u62;
-        ee = (double)(r.ej << 2) * sc.e62;
-    } else {
-        site_to_double(s);
-        const double rn = 1.0 / s.dM[0];
-        const double jx = s.dJ[0] * rn, jy = s.dJ[1] * rn, jz = D == 3 ? s.dJ[2] * rn : 0.0;
-        uu[0] = sc.u * jx;
-        uu[1] = sc.u * jy;
-        uu[2] = sc.u * jz;
-        ee = sc.e * (s.dE * rn - (jx * jx + jy * jy + jz * jz));
-    }
+    site_finish<D>(s, sc, uu, ee);
     const int64_t N = g.N, i = si.s;
     if (rho4)
 #pragma unroll

@@ -15,7 +15,7 @@ cudaError_t Launchers<D, Codec>::step(qlbm_ctx *h, bool odd)
 {
     if constexpr (std::is_same<Codec, CodecF64>::value) {
         cudaError_t e;
-        if (step_fix<D>(h, odd ? 1 : 0, h->pop, h->pop, &e)) return e;
+        if (step_fix<D>(h, odd ? 1 : 0, h->pop, h->pop, nullptr, &e)) return e;
     }
     const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
     const Planes<S, Q> pl = planes(h);
@@ -61,6 +61,25 @@ template <int D, class Codec>
 cudaError_t Launchers<D, Codec>::step_fd(qlbm_ctx *h, bool odd)
 {
     if constexpr (std::is_same<Codec, CodecF64>::value) {
+        // two kernels: the solve (one lane per site) writes the rebuilt density
+        // matrices, the fixed-point step reads them: 96 bytes per site and a
+        // second read of the state, against a solve held up by the one-kernel
+        // form's ~600 other double-precision instructions.  D3Q19 64^3: 677 ->
+        // 207 us.  Without room for the matrices, with a field, or at omega
+        // > 2: one kernel.
+        if (h->mag == FIELD_NONE && !h->fd_rho && cudaMalloc(&h->fd_rho, (size_t)h->g.N * sizeof(DQuad)) != cudaSuccess) {
+            cudaGetLastError();
+            h->fd_rho = nullptr;
+        }
+        FixConst fc;
+        if (h->mag == FIELD_NONE && h->fd_rho && make_fix_const(h->hc, h->dt / h->tau, &fc)) {
+            FdOut o{};
+            o.rho = static_cast<DQuad *>(h->fd_rho);
+            o.flags = h->flags;
+            cudaError_t e = fd_launch(h, o);
+            if (e == cudaSuccess) step_fix<D>(h, odd ? 1 : 0, h->pop, h->pop, h->fd_rho, &e);
+            return e;
+        }
         const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
         const FdArgs a{h->hc.beta0, h->hc.xi};
         return with_field(h->mag, [&](auto fc) {
