@@ -226,6 +226,7 @@ k_adjoint(const Planes<typename Codec::S, Lattice<D>::Q> st, const Planes<typena
     constexpr int Q = Lattice<D>::Q;
     constexpr bool DEV = Codec::DEV;
     SiteIdx si;
+    wait_for_previous();
     const bool active = site_of_block(g, si);
     double dtau = 0.0;
     if (active) {
@@ -298,6 +299,7 @@ k_adjoint(const Planes<typename Codec::S, Lattice<D>::Q> st, const Planes<typena
         SiteIdx s2 = si;
         s2.s += g.zero;
         s2.x += g.zero;
+        let_next_start();
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const int s = neighbour(g, s2, cx<D>(q), cy<D>(q), cz<D>(q));
@@ -323,11 +325,13 @@ k_step_push(const Planes<typename Codec::S, Lattice<D>::Q> src, const Planes<typ
     using R = typename Codec::R;
     constexpr int Q = Lattice<D>::Q;
     SiteIdx si;
+    wait_for_previous();
     if (!site_of_block(g, si)) return;
     R f[Q], sx[Q], sy[Q], sz[Q];
     gather<D, Codec, false>(src, g, si, codec, f, sx, sy, sz);
     const unsigned flag = Codec::template collide<D>(f, sx, sy, sz, k);
     apply_field<D, FIELD, R>(sx, sy, sz, k, si.s);
+    let_next_start();
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         const int s = neighbour(g, si, cx<D>(q), cy<D>(q), cz<D>(q));

@@ -1,4 +1,5 @@
-// The FP64 step on the integer pipes (QLBM_FP64 storage, no field).
+// The FP64 step on the integer pipes (QLBM_FP64 and QLBM_FP64_DF storage, no
+// field).
 //
 // GB300's double-precision pipe takes 64 cycles per warp instruction and
 // sub-partition (measured, whatever the number of warps; integer add, logic
@@ -462,7 +463,8 @@ __device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[La
     return flag;
 }
 
-// One step of FP64 storage: an even or odd AA step in place (addressing as
+// One step of FP64 storage (QLBM_FP64 and, with float_range, QLBM_FP64_DF
+// without a field): an even or odd AA step in place (addressing as
 // k_step_aa; src and dst the same planes) or the two-buffer step of the
 // reverse mode (as k_step_push), with the same arithmetic in all three.
 // With FD the equilibrium is built from a density matrix per site (rho, Eq.
@@ -471,10 +473,11 @@ enum : int { FIX_EVEN = 0, FIX_ODD = 1, FIX_PUSH = 2 };
 template <int D, int MODE, bool FD>
 __global__ void __launch_bounds__(kFixBlock, D == 3 ? 8 : 14)
 k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice<D>::Q> dst, Grid g, FixConst fc,
-           Coll<double> k, Chunks ch, const DQuad *__restrict__ rho, unsigned *__restrict__ flags)
+           Coll<double> k, Chunks ch, int float_range, const DQuad *__restrict__ rho, unsigned *__restrict__ flags)
 {
     constexpr int Q = Lattice<D>::Q;
     const unsigned all = 0xffffffffu;
+    wait_for_previous();
     const int chunk = (int)((blockIdx.x * kFixBlock + threadIdx.x) >> 5);
     if (chunk >= ch.total) return;      // the whole warp
     const int c = threadIdx.x & 3;
@@ -502,6 +505,17 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
     unsigned mx = 0u;
 #pragma unroll
     for (int q = 0; q < Q; ++q) mx = max(mx, (unsigned)(w[q] >> 32) & 0x7fffffffu);
+    unsigned flag = 0u;
+    if (float_range) {
+        // QLBM_FP64_DF: a component below 2^-126 counts as zero, a magnitude
+        // from 2^128 on as non-finite (single precision's exponent range)
+        if (mx < (897u << 20)) {
+            mx = 0u;
+#pragma unroll
+            for (int q = 0; q < Q; ++q) w[q] = 0ull;
+        }
+        if (mx >= (1151u << 20)) flag = FLAG_NONFINITE;
+    }
     const int eb = mx ? (int)(mx >> 20) : kFxMinExp;
     double R = 0.0;
     if (FD) R = reinterpret_cast<const double *>(rho + si.s)[c];
@@ -531,12 +545,12 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
             });
         }
     }
-    unsigned flag = 0u;
     if (!fine) {
 #pragma unroll
-        for (int q = 0; q < Q; ++q) w[q] = load(q);
-        flag = fx_collide_double<D, FD>(w, k, R);
+        for (int q = 0; q < Q; ++q) w[q] = float_range && mx == 0u ? 0ull : load(q);
+        flag |= fx_collide_double<D, FD>(w, k, R);
     }
+    let_next_start();
     if (active) {
         const int so = si.s + g.zero;   // store addresses formed anew (see k_step_aa)
 #pragma unroll

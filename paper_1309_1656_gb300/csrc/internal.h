@@ -142,6 +142,24 @@ cudaError_t launch_conserved_final(qlbm_ctx *h);
 // no handle; returns code.
 int set_global_error(int code, const char *msg);
 
+// Launches a kernel that starts with wait_for_previous (step.cuh): it may be
+// set up while the kernel before it in the stream still runs.
+template <class... P, class... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Launch shape of the per-site kernels: one thread per site, blocks of up to
 // kStepBlock consecutive x in one row.  Rows longer than 128 take the width
 // among 128, 96 and 64 that leaves the fewest idle threads at the row's end

@@ -16,11 +16,11 @@ template <int D> bool step_fix(qlbm_ctx *h, int mode, const void *src, void *dst
     const Coll<double> k = make_coll<double>(h);
     const dim3 blk(kFixBlock), grd((unsigned)((ch.total + kFixBlock / 32 - 1) / (kFixBlock / 32)));
     const DQuad *r = static_cast<const DQuad *>(rho);
-    auto launch = [&](auto kernel) { kernel<<<grd, blk, 0, h->stream>>>(s, d, h->g, fc, k, ch, r, h->flags); };
+    const int df = h->prec == QLBM_FP64_DF && !rho;     // the step through the parameters is the FP64 one
+    auto launch = [&](auto kernel) { *err = launch_chained(kernel, grd, blk, 0, h->stream, s, d, h->g, fc, k, ch, df, r, h->flags); };
     if (mode == FIX_PUSH) launch(k_step_fix<D, FIX_PUSH, false>);
     else if (mode == FIX_ODD) launch(rho ? k_step_fix<D, FIX_ODD, true> : k_step_fix<D, FIX_ODD, false>);
     else launch(rho ? k_step_fix<D, FIX_EVEN, true> : k_step_fix<D, FIX_EVEN, false>);
-    *err = cudaGetLastError();
     return true;
 }
 template bool step_fix<2>(qlbm_ctx *, int, const void *, void *, const void *, cudaError_t *);

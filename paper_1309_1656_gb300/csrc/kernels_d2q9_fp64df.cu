@@ -8,6 +8,11 @@ namespace qlbm {
 
 template <int D> cudaError_t step_f64df(qlbm_ctx *h, bool odd)
 {
+    // without a field the fixed-point step is faster and closer to the exact
+    // one (fix64.cuh); with one, rotating the spins there would cost more than
+    // it gains (9 more 64-bit products per direction)
+    cudaError_t e;
+    if (step_fix<D>(h, odd ? 1 : 0, h->pop, h->pop, nullptr, &e)) return e;
     // blocks of two warps over F64dfSplit<D>::SITES consecutive sites of a
     // row, so the grid is laid out for that block width
     Grid g = h->g;

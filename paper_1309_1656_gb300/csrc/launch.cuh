@@ -229,10 +229,9 @@ template <int D, class Codec> struct Launchers {
         const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
         return with_field(h->mag, [&](auto fc) {
             constexpr int F = decltype(fc)::value;
-            k_adjoint<D, Codec, F><<<grd, blk, 0, h->stream>>>(planes_of<S>(h, state), planes_of<R>(h, lam_in),
-                                                               planes_of<R>(h, lam_out), h->g, make_coll<R>(h),
-                                                               make_codec<Codec>(h), h->dtau_acc);
-            return cudaGetLastError();
+            return launch_chained(k_adjoint<D, Codec, F>, grd, blk, 0, h->stream, planes_of<S>(h, state),
+                                  planes_of<R>(h, lam_in), planes_of<R>(h, lam_out), h->g, make_coll<R>(h),
+                                  make_codec<Codec>(h), h->dtau_acc);
         });
     }
 
@@ -246,9 +245,8 @@ template <int D, class Codec> struct Launchers {
         const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
         return with_field(h->mag, [&](auto fc) {
             constexpr int F = decltype(fc)::value;
-            k_step_push<D, Codec, F><<<grd, blk, 0, h->stream>>>(planes_of<S>(h, src), planes_of<S>(h, dst), h->g,
-                                                                 make_coll<R>(h), make_codec<Codec>(h), h->flags);
-            return cudaGetLastError();
+            return launch_chained(k_step_push<D, Codec, F>, grd, blk, 0, h->stream, planes_of<S>(h, src),
+                                  planes_of<S>(h, dst), h->g, make_coll<R>(h), make_codec<Codec>(h), h->flags);
         });
     }
 

@@ -33,6 +33,18 @@ template <class S, int Q> struct Planes {
     typename QuadOf<S>::V *p[Q];
 };
 
+// Kernels that run back to back with their like (steps, the reverse sweep)
+// are launched as dependents of one another (launch_chained): such a kernel
+// touches memory only once its predecessor has finished (wait_for_previous),
+// and its successor is set up when all its blocks have reached their stores
+// (let_next_start; at the kernels' start instead, the successor's waiting
+// blocks get in the way: 64 x 64 FP64 3.07 us per step, D3Q19 32^3 FP32 4.9).
+// Without effect next to other work.  Per step, before -> after: D2Q9 64^2
+// FP64 2.64 -> 2.25 us, D2Q9 256^2 FP64 10.1 -> 9.7, D3Q19 128^3 FP16 102.8 ->
+// 100.0, FP32 186.6 -> 184.3.
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Site of the calling thread; false if it lies beyond the row.
 struct SiteIdx {
     int x, y, z;
@@ -132,6 +144,7 @@ k_step_aa(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Coll<typena
     using R = typename Codec::R;
     constexpr int Q = Lattice<D>::Q;
     SiteIdx si;
+    wait_for_previous();
     if (!site_of_block(g, si)) return;
     R f[Q], sx[Q], sy[Q], sz[Q];
     gather<D, Codec, ODD>(pl, g, si, codec, f, sx, sy, sz);
@@ -143,6 +156,7 @@ k_step_aa(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Coll<typena
     SiteIdx so = si;
     so.s += g.zero;
     so.x += g.zero;
+    let_next_start();
 #pragma unroll
     for (int q = 0; q < Q; ++q) {
         // population q goes to slot opposite(q) at x (even) or slot q at x + e_q (odd)
@@ -230,6 +244,7 @@ k_step_aa_rows(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Coll<t
     using V = typename QuadOf<typename Codec::S>::V;
     constexpr int Q = Lattice<D>::Q;
     extern __shared__ __align__(16) unsigned char rows_smem[];
+    wait_for_previous();
     const int bw = blockDim.x;
     // stage t, slot q of this thread at mine[(t * Q + q) * bw]
     V *mine = reinterpret_cast<V *>(rows_smem) + threadIdx.x;
@@ -265,6 +280,7 @@ k_step_aa_rows(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Coll<t
         }
         flag |= Codec::template collide<D>(f, sx, sy, sz, k);
         apply_field<D, FIELD, R>(sx, sy, sz, k, cur.s);
+        if (row + 1 == rend) let_next_start();
         // store addresses recomputed from g.zero (see k_step_aa)
         const int so = cur.s + g.zero;
 #pragma unroll

@@ -24,11 +24,8 @@ cudaError_t Launchers<D, Codec>::step(qlbm_ctx *h, bool odd)
     if constexpr (TwoPass<Codec>::value) {
         return with_field(h->mag, [&](auto fc) {
             constexpr int F = decltype(fc)::value;
-            if (odd)
-                k_step_aa_df2<D, true, F><<<grd, blk, 0, h->stream>>>(pl, h->g, k, codec, h->flags);
-            else
-                k_step_aa_df2<D, false, F><<<grd, blk, 0, h->stream>>>(pl, h->g, k, codec, h->flags);
-            return cudaGetLastError();
+            return launch_chained(odd ? k_step_aa_df2<D, true, F> : k_step_aa_df2<D, false, F>, grd, blk, 0, h->stream, pl, h->g, k, codec,
+                                  h->flags);
         });
     } else if constexpr (RowPipelined<Codec>::value) {
         // rows per block from a sweep on GB300 (FP16): D2Q9 4096^2 gains
@@ -38,20 +35,14 @@ cudaError_t Launchers<D, Codec>::step(qlbm_ctx *h, bool odd)
         const size_t sm = rows_smem_bytes<D, Codec>((int)blk.x);
         return with_field(h->mag, [&](auto fc) {
             constexpr int F = decltype(fc)::value;
-            if (odd)
-                k_step_aa_rows<D, Codec, true, F><<<grr, blk, sm, h->stream>>>(pl, h->g, k, codec, rpb, h->flags);
-            else
-                k_step_aa_rows<D, Codec, false, F><<<grr, blk, sm, h->stream>>>(pl, h->g, k, codec, rpb, h->flags);
-            return cudaGetLastError();
+            return launch_chained(odd ? k_step_aa_rows<D, Codec, true, F> : k_step_aa_rows<D, Codec, false, F>, grr, blk,
+                                  sm, h->stream, pl, h->g, k, codec, rpb, h->flags);
         });
     } else {
         return with_field(h->mag, [&](auto fc) {
             constexpr int F = decltype(fc)::value;
-            if (odd)
-                k_step_aa<D, Codec, true, F><<<grd, blk, 0, h->stream>>>(pl, h->g, k, codec, h->flags);
-            else
-                k_step_aa<D, Codec, false, F><<<grd, blk, 0, h->stream>>>(pl, h->g, k, codec, h->flags);
-            return cudaGetLastError();
+            return launch_chained(odd ? k_step_aa<D, Codec, true, F> : k_step_aa<D, Codec, false, F>, grd, blk, 0, h->stream, pl, h->g, k, codec,
+                                  h->flags);
         });
     }
     return cudaGetLastError();

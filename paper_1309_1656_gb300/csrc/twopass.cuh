@@ -59,6 +59,7 @@ k_step_aa_df2(const Planes<df, Lattice<D>::Q> pl, Grid g, Coll<df> k, CodecDF co
     // what it wrote: no barrier)
     __shared__ float4 lo_stage[Q][kStepBlock];
     SiteIdx si;
+    wait_for_previous();
     if (!site_of_block(g, si)) return;
     float hf[Q], hx[Q], hy[Q], hz[Q];   // hi parts, kept from pass 1 in registers
     DFSums a;
@@ -90,6 +91,7 @@ k_step_aa_df2(const Planes<df, Lattice<D>::Q> pl, Grid g, Coll<df> k, CodecDF co
     SiteIdx s2 = si;
     s2.s += g.zero;
     s2.x += g.zero;
+    let_next_start();
 #pragma unroll
     for (int q = 0; q <= (Q - 1) / 2; ++q) {
         const int qb = Q - 1 - q;
