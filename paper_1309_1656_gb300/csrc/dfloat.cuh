@@ -106,7 +106,7 @@ __device__ __forceinline__ df dfma(df a, df b, df c)
 // pieces so that the two-pass kernel can stream the populations through the
 // moment sums (df_accumulate), form the per-site coefficients
 // (df_coefficients) and update a direction together with its opposite
-// (df_pair):
+// (df_pair_h, df_update):
 // W' = (1 - omega) W + omega w_i P_i rho, with P_{+-} = bq + c4 t^2 +- c3 t
 // for the pair's t = +-(i.j).
 // A running sum of double-float terms: the hi parts are added exactly
@@ -232,50 +232,63 @@ template <int D> __device__ __forceinline__ DFCoef df_coefficients(const DFSums 
                                  a.e1.value() + scale2(a.e2.value(), 2.f), k);
 }
 
-// Updates direction q (q <= (Q-1)/2) and its opposite Q-1-q in place; for
-// the rest direction (the middle index) only the first set is used.
+// omega w_i P_i = hp for direction q (q <= (Q-1)/2), hm for its opposite
+// Q-1-q (the rest direction, the middle index, has hp only), without omega.
 template <int D>
-__device__ __forceinline__ void df_pair(const DFCoef &c, const Coll<df> &k, int q, df &f, df &x, df &y, df &z,
-                                        df &fb, df &xb, df &yb, df &zb)
+__device__ __forceinline__ void df_pair_h(const DFCoef &c, const Coll<df> &k, int q, df &hp, df &hm)
 {
-    constexpr int Q = Lattice<D>::Q;
     const int cls = cnorm2<D>(q);
-    df hp, hm;
     if (cls == 0) {
         hp = hm = k.w[0] * c.bq[0];
-    } else {
-        df t(0.f, 0.f);
-        bool first = true;
-        if (cx<D>(q)) {
-            t = scale2(c.jx, (float)cx<D>(q));
-            first = false;
-        }
-        if (cy<D>(q)) {
-            t = first ? scale2(c.jy, (float)cy<D>(q)) : t + scale2(c.jy, (float)cy<D>(q));
-            first = false;
-        }
-        if (cz<D>(q)) t = first ? scale2(c.jz, (float)cz<D>(q)) : t + scale2(c.jz, (float)cz<D>(q));
-        const df A = dfma(k.c4, t * t, c.bq[cls]);
-        const df B = k.c3 * t;
-        hp = k.w[cls] * (A + B);
-        hm = k.w[cls] * (A - B);
+        return;
     }
-    f = dfma(hp, c.on, c.omc * f);
-    x = dfma(hp, c.oSx, c.omc * x);
-    y = dfma(hp, c.oSy, c.omc * y);
-    z = dfma(hp, c.oSz, c.omc * z);
-    if (Q - 1 - q != q) {
-        fb = dfma(hm, c.on, c.omc * fb);
-        xb = dfma(hm, c.oSx, c.omc * xb);
-        yb = dfma(hm, c.oSy, c.omc * yb);
-        zb = dfma(hm, c.oSz, c.omc * zb);
+    df t(0.f, 0.f);
+    bool first = true;
+    if (cx<D>(q)) {
+        t = scale2(c.jx, (float)cx<D>(q));
+        first = false;
     }
+    if (cy<D>(q)) {
+        t = first ? scale2(c.jy, (float)cy<D>(q)) : t + scale2(c.jy, (float)cy<D>(q));
+        first = false;
+    }
+    if (cz<D>(q)) t = first ? scale2(c.jz, (float)cz<D>(q)) : t + scale2(c.jz, (float)cz<D>(q));
+    const df A = dfma(k.c4, t * t, c.bq[cls]);
+    const df B = k.c3 * t;
+    hp = k.w[cls] * (A + B);
+    hm = k.w[cls] * (A - B);
+}
+
+// W' = (1 - omega) W + h omega (n, S) of one population.
+__device__ __forceinline__ void df_update(const DFCoef &c, df h, df &f, df &x, df &y, df &z)
+{
+    f = dfma(h, c.on, c.omc * f);
+    x = dfma(h, c.oSx, c.omc * x);
+    y = dfma(h, c.oSy, c.omc * y);
+    z = dfma(h, c.oSz, c.omc * z);
+}
+
+// a0 x0 + a1 x1 + a2 x2 + a3 x3 with each product exact to ~2^-48 (Dekker),
+// three TwoSums of the leading parts and one of the result.
+__device__ __forceinline__ df dot4(df a0, df x0, df a1, df x1, df a2, df x2, df a3, df x3)
+{
+    const float p0 = __fmul_rn(a0.hi, x0.hi), p1 = __fmul_rn(a1.hi, x1.hi), p2 = __fmul_rn(a2.hi, x2.hi),
+                p3 = __fmul_rn(a3.hi, x3.hi);
+    float e0 = __fmaf_rn(a0.hi, x0.hi, -p0), e1 = __fmaf_rn(a1.hi, x1.hi, -p1), e2 = __fmaf_rn(a2.hi, x2.hi, -p2),
+          e3 = __fmaf_rn(a3.hi, x3.hi, -p3);
+    e0 = __fmaf_rn(a0.hi, x0.lo, __fmaf_rn(a0.lo, x0.hi, e0));
+    e1 = __fmaf_rn(a1.hi, x1.lo, __fmaf_rn(a1.lo, x1.hi, e1));
+    e2 = __fmaf_rn(a2.hi, x2.lo, __fmaf_rn(a2.lo, x2.hi, e2));
+    e3 = __fmaf_rn(a3.hi, x3.lo, __fmaf_rn(a3.lo, x3.hi, e3));
+    const df s = two_sum(p0, p1), t = two_sum(p2, p3), u = two_sum(s.hi, t.hi);
+    const float lo = __fadd_rn(__fadd_rn(u.lo, __fadd_rn(s.lo, t.lo)), __fadd_rn(__fadd_rn(e0, e1), __fadd_rn(e2, e3)));
+    return two_sum(u.hi, lo);
 }
 
 // Double-float storage: each value a pair of floats (8 bytes, like a
 // double; 48-bit significand) in the split hi / lo layout above.  Its step
 // is the two-pass kernel of twopass.cuh (df_accumulate, df_coefficients,
-// df_pair); the codec itself only moves values.
+// df_pair_h, df_update); the codec itself only moves values.
 struct CodecDF {
     using S = df;
     using V = QuadOf<S>::V;

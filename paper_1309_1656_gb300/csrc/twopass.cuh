@@ -29,14 +29,19 @@ template <> struct TwoPass<CodecDF> {
     template <int D> static constexpr int min_blocks() { return D == 2 ? 5 : 4; }
 };
 
-// Spin rotation of the magnetic-field term for one population (see
-// rotate_spins).
-__device__ __forceinline__ void rotate_one(df &x, df &y, df &z, const df (&r)[9])
+// A population's update with the magnetic-field term: the rotation r of
+// (1 - omega) s + h omega S taken as (1 - omega) r s + h (r omega S), m =
+// (1 - omega) r and the rotated omega S (in c) formed once per site, one
+// four-term product sum per component.  Updated first and rotated then, it
+// takes 22 + 43 single-precision operations per component, this 46 (D2Q9
+// 1501 x 777, uniform field: 146 -> 132 us per step).
+__device__ __forceinline__ void df_update_rotated(const DFCoef &c, df h, const df (&m)[9], df &f, df &x, df &y, df &z)
 {
-    const df a = x, b = y, c = z;
-    x = r[0] * a + r[1] * b + r[2] * c;
-    y = r[3] * a + r[4] * b + r[5] * c;
-    z = r[6] * a + r[7] * b + r[8] * c;
+    f = dfma(h, c.on, c.omc * f);
+    const df a = x, b = y, d = z;
+    x = dot4(m[0], a, m[1], b, m[2], d, h, c.oSx);
+    y = dot4(m[3], a, m[4], b, m[5], d, h, c.oSy);
+    z = dot4(m[6], a, m[7], b, m[8], d, h, c.oSz);
 }
 
 // Location of population p of site si: slot and site index.
@@ -75,16 +80,27 @@ k_step_aa_df2(const Planes<df, Lattice<D>::Q> pl, Grid g, Coll<df> k, CodecDF co
         lo_stage[p][threadIdx.x] = l;
         df_accumulate<D>(a, p, df(h.x, l.x), df(h.y, l.y), df(h.z, l.z), df(h.w, l.w));
     }
-    const DFCoef c = df_coefficients<D>(a, k);
-    // a per-site field: the site's rotation, formed in double from its unit
-    // quaternion and rounded to double-float pairs
-    df rs[9];
-    if constexpr (FIELD == FIELD_SITE) {
-        double w, x, y, z, r[9];
-        load_quat(k.qf + si.s, w, x, y, z);
-        quat_rotation(w, x, y, z, r);
+    DFCoef c = df_coefficients<D>(a, k);
+    // the field's rotation: the uniform one, or the site's own, formed in
+    // double from its unit quaternion and rounded to double-float pairs
+    df rm[9];
+    if constexpr (FIELD != FIELD_NONE) {
+        if constexpr (FIELD == FIELD_SITE) {
+            double w, x, y, z, r[9];
+            load_quat(k.qf + si.s, w, x, y, z);
+            quat_rotation(w, x, y, z, r);
 #pragma unroll
-        for (int i = 0; i < 9; ++i) rs[i] = df(r[i]);
+            for (int i = 0; i < 9; ++i) rm[i] = df(r[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 9; ++i) rm[i] = k.rot[i];
+        }
+        const df Sx = c.oSx, Sy = c.oSy, Sz = c.oSz;
+        c.oSx = rm[0] * Sx + rm[1] * Sy + rm[2] * Sz;
+        c.oSy = rm[3] * Sx + rm[4] * Sy + rm[5] * Sz;
+        c.oSz = rm[6] * Sx + rm[7] * Sy + rm[8] * Sz;
+#pragma unroll
+        for (int i = 0; i < 9; ++i) rm[i] = c.omc * rm[i];
     }
     // g.zero (0 at run time) makes pass 2's addresses distinct expressions,
     // so the compiler re-loads the lo parts instead of keeping pass 1's.
@@ -107,13 +123,14 @@ k_step_aa_df2(const Planes<df, Lattice<D>::Q> pl, Grid g, Coll<df> k, CodecDF co
             yb = df(hy[qb], lb.z);
             zb = df(hz[qb], lb.w);
         }
-        df_pair<D>(c, k, q, f, x, y, z, fb, xb, yb, zb);
-        if constexpr (FIELD == FIELD_UNIFORM) {
-            rotate_one(x, y, z, k.rot);
-            if (qb != q) rotate_one(xb, yb, zb, k.rot);
-        } else if constexpr (FIELD == FIELD_SITE) {
-            rotate_one(x, y, z, rs);
-            if (qb != q) rotate_one(xb, yb, zb, rs);
+        df hp, hm;
+        df_pair_h<D>(c, k, q, hp, hm);
+        if constexpr (FIELD == FIELD_NONE) {
+            df_update(c, hp, f, x, y, z);
+            if (qb != q) df_update(c, hm, fb, xb, yb, zb);
+        } else {
+            df_update_rotated(c, hp, rm, f, x, y, z);
+            if (qb != q) df_update_rotated(c, hm, rm, fb, xb, yb, zb);
         }
         // population p goes to slot opposite(p) at x (even) or slot p at x + e_p (odd)
         codec.store4(pl.p[ODD ? q : qb] + (ODD ? neighbour(g, s2, cx<D>(q), cy<D>(q), cz<D>(q)) : s2.s), f, x, y,
