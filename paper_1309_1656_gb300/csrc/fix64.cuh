@@ -1,5 +1,4 @@
-// The FP64 step on the integer pipes (QLBM_FP64 and QLBM_FP64_DF storage, no
-// field).
+// The FP64 step on the integer pipes (QLBM_FP64 and QLBM_FP64_DF storage).
 //
 // GB300's double-precision pipe takes 64 cycles per warp instruction and
 // sub-partition (measured, whatever the number of warps; integer add, logic
@@ -155,6 +154,7 @@ struct FixConst {
     FxSplit ga[2];          // q62, rest and axis class
     FxSplit c3, c4;         // q62
     long long d0;           // q60
+    int valid;              // 0: every site in double
 };
 constexpr long long kFxOne = 1LL << 62;   // 1.0 in q62
 
@@ -162,6 +162,7 @@ constexpr long long kFxOne = 1LL << 62;   // 1.0 in q62
 // value that the fixed-point step takes (no result near the ends of the
 // double range; below the 1e30 that the step flags as non-finite).
 constexpr int kFxMinExp = 128, kFxMaxExp = 1023 + 90;
+constexpr int kFxZeroExp = 2000;    // aligned to this exponent everything is shifted out
 
 // The double with words (hi, lo) in units of 2^(eb - 1080), truncated.
 FX_FN long long fx_align(unsigned hi, unsigned lo, int eb)
@@ -354,6 +355,7 @@ inline Dd reciprocal(Dd a)
 // double-precision kernel steps the lattice).
 inline bool make_fix_const(const HostConsts &k, double omega, FixConst *o)
 {
+    *o = FixConst{};
     if (!(omega > 0.0 && omega <= 2.0)) return false;
     bool ok = k.w[2] * (k.d == 3 ? 2.0 : 4.0) == k.w[1];     // the diagonal class is shifts of the axis class
     auto fix = [&](Dd v, double scale, double lim) {
@@ -378,6 +380,7 @@ inline bool make_fix_const(const HostConsts &k, double omega, FixConst *o)
     o->c3 = fx_split(fix(c3, q62, 1.99));
     o->c4 = fx_split(fix(c4, q62, 1.99));
     o->d0 = fix(c * reciprocal(K), q62 / 4.0, 2.0);
+    o->valid = ok;
     return ok;
 }
 
@@ -419,13 +422,69 @@ __device__ __forceinline__ long long fx_from_lane0(long long v)
     return __shfl_sync(0xffffffffu, v, 0, 4);   // the site's lane 0 (component f)
 }
 
+// The magnetic-field term: the rotation of the spins by the unit quaternion
+// (w, x, y, z) (FIELD_UNIFORM: uq, FIELD_SITE: of site s).  Lane c = 1..3 holds
+// component c; in cyclic order p, q, r = its own component of the vector part,
+// the next and the one after, its row of the rotation matrix is
+//   1 - 2 (q^2 + r^2)  (own),  2 (p q - w r)  (next),  2 (p r + w q)  (after).
+// For the uniform field the host gives each lane's row (in the same order) in
+// q62 and (1 - omega) times it; row 0 is the identity's.
+struct FixField {
+    double v[4];        // (w, x, y, z)
+    FxSplit r[4][3], m[4][3];
+};
+inline void make_fix_field(const double (&rot)[9], const double (&quat)[4], double omega, FixField *o)
+{
+    auto q62 = [](Dd v) { return fx_split(llrint(v.h * 4611686018427387904.0) + llrint(v.l * 4611686018427387904.0)); };
+    const Dd omc = Dd(1.0) + Dd(-omega);
+    for (int i = 0; i < 4; ++i) o->v[i] = quat[i];
+    for (int c = 0; c < 4; ++c)
+        for (int b = 0; b < 3; ++b) {
+            const double r = c ? rot[3 * (c - 1) + (c - 1 + b) % 3] : (b ? 0.0 : 1.0);
+            o->r[c][b] = q62(Dd(r));
+            o->m[c][b] = q62(omc * Dd(r));
+        }
+}
+FX_FN int fx_next_lane(int c) { return c == 3 ? 1 : c + 1; }
+FX_FN int fx_prev_lane(int c) { return c <= 1 ? 3 : c - 1; }
+template <int FIELD>
+__device__ __forceinline__ void fx_load_quat(const FixField &uq, const DQuad *qf, int s, int c, double (&o)[4])
+{
+    const int p = c ? c : 1;
+    const double *v = FIELD == FIELD_SITE ? reinterpret_cast<const double *>(qf + s) : uq.v;
+    o[0] = v[0];
+    o[1] = v[p];
+    o[2] = v[fx_next_lane(p)];
+    o[3] = v[fx_prev_lane(p)];
+}
+// A number of magnitude <= 1 in q62.
+__device__ __forceinline__ FxSplit fx_unit(double v)
+{
+    return fx_split(fx_align((unsigned)__double2hiint(v), (unsigned)__double2loint(v), 1023) << 5);
+}
+// The row of the rotation matrix (q62); lane 0: the identity's.
+__device__ __forceinline__ void fx_rotation_row(const double (&fq)[4], int c, FxSplit (&R)[3])
+{
+    const FxSplit w = fx_unit(fq[0]), p = fx_unit(fq[1]), q = fx_unit(fq[2]), r = fx_unit(fq[3]);
+    const long long d = kFxOne - 8 * (fx_mul(q, q) + fx_mul(r, r));     // q60 products
+    const long long n = 8 * (fx_mul(p, q) - fx_mul(w, r)), a = 8 * (fx_mul(p, r) + fx_mul(w, q));
+    R[0] = fx_split(c ? d : kFxOne);
+    R[1] = fx_split(c ? n : 0);
+    R[2] = fx_split(c ? a : 0);
+}
+__device__ __forceinline__ FxSplit fx_shfl(FxSplit v, int lane)
+{
+    return FxSplit{__shfl_sync(0xffffffffu, v.hi, lane, 4), __shfl_sync(0xffffffffu, v.lo, lane, 4)};
+}
+
 // The step of one component in double (collide's formulas), for warps with a
 // site outside the fixed-point form; lane c = 0 holds f, 1..3 the spins.
 // FD: the equilibrium is built from the component R of a rebuilt density
-// matrix instead of M (the flag then looks at n only).
-template <int D, bool FD>
+// matrix instead of M (the flag then looks at n only).  FIELD: the spins are
+// rotated by the unit quaternion fq (fx_load_quat).
+template <int D, bool FD, bool FIELD>
 __device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[Lattice<D>::Q], const Coll<double> &k,
-                                                      double R)
+                                                      double R, const double (&fq)[4])
 {
     constexpr int Q = Lattice<D>::Q;
     double M = 0.0, J[3] = {0.0, 0.0, 0.0}, E = 0.0;
@@ -454,6 +513,17 @@ __device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[La
         const double h = k.w[cnorm2<D>(q)] * fma(t, fma(k.c4, t, k.c3), bq[cnorm2<D>(q)]);
         w[q] = (unsigned long long)__double_as_longlong(fma(k.omega, fma(h, FD ? R : M, -v), v));
     }
+    if constexpr (FIELD) {
+        const int c = threadIdx.x & 3;
+        const double r0 = 1.0 - 2.0 * (fq[2] * fq[2] + fq[3] * fq[3]), r1 = 2.0 * (fq[1] * fq[2] - fq[0] * fq[3]),
+                     r2 = 2.0 * (fq[1] * fq[3] + fq[0] * fq[2]);
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            const double v = __longlong_as_double((long long)w[q]);
+            const double v1 = __shfl_sync(all, v, fx_next_lane(c), 4), v2 = __shfl_sync(all, v, fx_prev_lane(c), 4);
+            if (c) w[q] = (unsigned long long)__double_as_longlong(r0 * v + r1 * v1 + r2 * v2);
+        }
+    }
     double sum = (threadIdx.x & 3) ? fabs(M) : fabs(be);
     sum += __shfl_xor_sync(all, sum, 1, 4);
     sum += __shfl_xor_sync(all, sum, 2, 4);
@@ -463,17 +533,29 @@ __device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[La
     return flag;
 }
 
-// One step of FP64 storage (QLBM_FP64 and, with float_range, QLBM_FP64_DF
-// without a field): an even or odd AA step in place (addressing as
-// k_step_aa; src and dst the same planes) or the two-buffer step of the
-// reverse mode (as k_step_push), with the same arithmetic in all three.
+// One step of FP64 storage (QLBM_FP64 and QLBM_FP64_DF): an
+// even or odd AA step in place (addressing as k_step_aa; src and dst the same
+// planes) or the two-buffer step of the reverse mode (as k_step_push), with
+// the same arithmetic in all three.
 // With FD the equilibrium is built from a density matrix per site (rho, Eq.
 // WeqDiscr) instead of the populations' own; P_i keeps their u and eps.
+// With a field the three spin components share one alignment (|X| < 2^57, so
+// that a rotated sum still fits) and the rotation R is folded into the
+// relaxation: sum_b (1 - omega) R_ab X_b + h (R M)_a, the other two components
+// from the neighbouring lanes.
+// rg: the largest high word (magnitude) of a component that counts as zero,
+// and the smallest that is non-finite; QLBM_FP64_DF has single precision's
+// exponent range there (2^-126, 2^128).
+struct FixRange {
+    unsigned zero, bad;
+};
+inline FixRange make_fix_range(bool single) { return single ? FixRange{(897u << 20) - 1u, 1151u << 20} : FixRange{0u, ~0u}; }
 enum : int { FIX_EVEN = 0, FIX_ODD = 1, FIX_PUSH = 2 };
-template <int D, int MODE, bool FD>
+template <int D, int MODE, bool FD, int FIELD>
 __global__ void __launch_bounds__(kFixBlock, D == 3 ? 8 : 14)
 k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice<D>::Q> dst, Grid g, FixConst fc,
-           Coll<double> k, Chunks ch, int float_range, const DQuad *__restrict__ rho, unsigned *__restrict__ flags)
+           Coll<double> k, Chunks ch, FixRange rg, const DQuad *__restrict__ rho, FixField uq,
+           unsigned *__restrict__ flags)
 {
     constexpr int Q = Lattice<D>::Q;
     const unsigned all = 0xffffffffu;
@@ -505,21 +587,20 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
     unsigned mx = 0u;
 #pragma unroll
     for (int q = 0; q < Q; ++q) mx = max(mx, (unsigned)(w[q] >> 32) & 0x7fffffffu);
-    unsigned flag = 0u;
-    if (float_range) {
-        // QLBM_FP64_DF: a component below 2^-126 counts as zero, a magnitude
-        // from 2^128 on as non-finite (single precision's exponent range)
-        if (mx < (897u << 20)) {
-            mx = 0u;
-#pragma unroll
-            for (int q = 0; q < Q; ++q) w[q] = 0ull;
-        }
-        if (mx >= (1151u << 20)) flag = FLAG_NONFINITE;
+    unsigned flag = mx >= rg.bad ? FLAG_NONFINITE : 0u;
+    if constexpr (FIELD != FIELD_NONE) {
+        const unsigned m1 = __shfl_sync(all, mx, 1, 4), m2 = __shfl_sync(all, mx, 2, 4), m3 = __shfl_sync(all, mx, 3, 4);
+        if (c) mx = max(m1, max(m2, m3));
     }
-    const int eb = mx ? (int)(mx >> 20) : kFxMinExp;
+    // a component that counts as zero is shifted out altogether (eb); with a
+    // field the spins have one bit of headroom
+    const bool zero = mx <= rg.zero;
+    const int eb = zero ? kFxZeroExp : (int)(mx >> 20) + (FIELD != FIELD_NONE && c ? 1 : 0);
+    double fq[4] = {1.0, 0.0, 0.0, 0.0};
+    if constexpr (FIELD != FIELD_NONE) fx_load_quat<FIELD>(uq, k.qf, si.s, c, fq);
     double R = 0.0;
     if (FD) R = reinterpret_cast<const double *>(rho + si.s)[c];
-    bool fine = __all_sync(all, eb >= kFxMinExp && eb <= kFxMaxExp);
+    bool fine = fc.valid && __all_sync(all, zero || (eb >= kFxMinExp && eb <= kFxMaxExp));
     if (fine) {
         long long X[Q], M, J[3], E;
 #pragma unroll
@@ -533,22 +614,52 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
         if (fine) {
             if (FD) {       // rho's component in the units of M
                 const int rh = __double2hiint(R), e = (rh >> 20) & 0x7ff;
-                const bool zero = e <= eb - 70;     // below U / 2^13
-                fine = __all_sync(all, zero || (e < eb + 5 && mx != 0u));
-                M = zero ? 0 : __double2ll_rn(__hiloint2double(rh + (1080 - eb) * (1 << 20), __double2loint(R)));
+                const bool none = e <= eb - 70;     // below U / 2^13
+                fine = __all_sync(all, none || (e < eb + 5 && !zero));
+                M = none ? 0 : __double2ll_rn(__hiloint2double(rh + (1080 - eb) * (1 << 20), __double2loint(R)));
             }
-            const FxSplit m = fx_split(M);
             const int shift = (eb - 1078) * (1 << 20);
-            fx_each_h<D>(cf, [&](int q, long long h) {
-                w[q] = (unsigned long long)__double_as_longlong(
-                    fx_to_double(fx_update(X[q], fc.omc, h, m), shift));
-            });
+            if constexpr (FIELD == FIELD_NONE) {
+                const FxSplit m = fx_split(M);
+                fx_each_h<D>(cf, [&](int q, long long h) {
+                    w[q] = (unsigned long long)__double_as_longlong(
+                        fx_to_double(fx_update(X[q], fc.omc, h, m), shift));
+                });
+            } else {
+                const int n1 = fx_next_lane(c), n2 = fx_prev_lane(c);
+                FxSplit r[3];
+                if constexpr (FIELD == FIELD_SITE) {
+                    fx_rotation_row(fq, c, r);
+                } else {
+#pragma unroll
+                    for (int b = 0; b < 3; ++b) r[b] = uq.r[c][b];
+                }
+                FxSplit m = fx_split(M);
+                const FxSplit m1 = fx_shfl(m, n1), m2 = fx_shfl(m, n2);
+                if (c) m = fx_split((fx_mul(r[0], m) + fx_mul(r[1], m1) + fx_mul(r[2], m2) + 1) << 2);
+#pragma unroll
+                for (int b = 0; b < 3; ++b) {
+                    if constexpr (FIELD == FIELD_SITE)
+                        r[b] = c ? fx_split(fx_mul(fc.omc, r[b]) << 2) : (b ? FxSplit{0, 0} : fc.omc);
+                    else
+                        r[b] = uq.m[c][b];
+                }
+                fx_each_h<D>(cf, [&](int q, long long h) {
+                    const FxSplit x = fx_split(X[q]), x1 = fx_shfl(x, n1), x2 = fx_shfl(x, n2), g = fx_split(h);
+                    long long t = fx_mad(x.hi, r[0].lo, fx_mad(x.lo, r[0].hi, 0x80000000LL));
+                    t = fx_mad(x1.hi, r[1].lo, fx_mad(x1.lo, r[1].hi, t));
+                    t = fx_mad(x2.hi, r[2].lo, fx_mad(x2.lo, r[2].hi, t));
+                    t = fx_mad(m.hi, g.lo, fx_mad(m.lo, g.hi, t)) >> 32;
+                    t = fx_mad(x2.hi, r[2].hi, fx_mad(x1.hi, r[1].hi, fx_mad(x.hi, r[0].hi, t)));
+                    w[q] = (unsigned long long)__double_as_longlong(fx_to_double(fx_mad(m.hi, g.hi, t), shift));
+                });
+            }
         }
     }
     if (!fine) {
 #pragma unroll
-        for (int q = 0; q < Q; ++q) w[q] = float_range && mx == 0u ? 0ull : load(q);
-        flag |= fx_collide_double<D, FD>(w, k, R);
+        for (int q = 0; q < Q; ++q) w[q] = zero ? 0ull : load(q);
+        flag |= fx_collide_double<D, FD, FIELD != FIELD_NONE>(w, k, R, fq);
     }
     let_next_start();
     if (active) {

@@ -67,6 +67,7 @@ struct qlbm_ctx {
     int mag = 0;                        // magnetic-field term: FIELD_NONE, FIELD_UNIFORM or FIELD_SITE
     void *qfield = nullptr;             // per-site field: N unit quaternions (float4, or DQuad for FP64)
     double rot[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};   // its per-step spin rotation
+    double quat[4] = {1, 0, 0, 0};      // the same as a unit quaternion
     unsigned long long *fd_fail = nullptr;   // device counter of unresolved sites
     void *fd_rho = nullptr;             // density matrices of the step through the parameters (DQuad per site)
     unsigned long long *neg_count = nullptr; // device counter of the negative-equilibrium diagnostic
@@ -115,13 +116,13 @@ const LatticeOps *ops_d3q19_fp16();
 const LatticeOps *ops_d3q19_df64();
 const LatticeOps *ops_d2q9_fp64df();
 const LatticeOps *ops_d3q19_fp64df();
-// the double-float step on FP64 storage (kernels_<lattice>_fp64df.cu)
+// the step of QLBM_FP64_DF (kernels_<lattice>_fp64_fix.cu)
 template <int D> cudaError_t step_f64df(qlbm_ctx *h, bool odd);
 // The FP64 step on the integer pipes (kernels_<lattice>_fp64_fix.cu): mode 0
 // even AA step, 1 odd, 2 two-buffer step from src to dst; rho: the density
 // matrices (DQuad per site) the equilibrium is built from, or NULL for the
-// populations' own.  False, with nothing launched, where it does not apply (a
-// magnetic field; omega > 2).
+// populations' own.  False, with nothing launched, where it does not apply
+// (QLBM_FP64 with omega > 2).
 template <int D> bool step_fix(qlbm_ctx *h, int mode, const void *src, void *dst, const void *rho, cudaError_t *err);
 
 inline const LatticeOps *lattice_ops(int d, int prec)

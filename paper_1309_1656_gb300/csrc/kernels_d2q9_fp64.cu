@@ -1,5 +1,5 @@
 // D2Q9 (Sec. 3.1, d = 2, b = 9) kernels for FP64 storage: the dispatch tables of FP64 storage with the
-// FP64 and the double-float step, in a translation unit of its own so the instantiations
+// FP64 step and QLBM_FP64_DF's, in a translation unit of its own so the instantiations
 // compile in parallel.
 #include "steplaunch.cuh"
 
@@ -8,9 +8,8 @@ template cudaError_t Launchers<2, CodecF64>::step(qlbm_ctx *, bool);
 template cudaError_t Launchers<2, CodecF64>::step_fd(qlbm_ctx *, bool);
 const LatticeOps *ops_d2q9_fp64() { return Launchers<2, CodecF64>::table(); }
 
-// FP64 storage with the double-float step: the FP64 operations, the step of
-// kernels_d2q9_fp64df.cu, no reverse mode (its recorded trajectory would
-// come from the FP64 step).
+// QLBM_FP64_DF: the FP64 operations, the fixed-point step with single
+// precision's exponent range (kernels_d2q9_fp64_fix.cu), no reverse mode.
 const LatticeOps *ops_d2q9_fp64df()
 {
     static const LatticeOps t = [] {

@@ -35,8 +35,8 @@ def worst(got, exp):
     return max(float(np.max(np.abs(got[:, c] - exp[:, c])) / max(np.max(np.abs(exp[:, c])), 1e-300)) for c in range(4))
 
 
-def reference(q, d, dims, tau, st, n, dt=1.0):
-    """n steps in long double (Eqs. DiscrAvr, WeqAlgo, CollisionStep, TransportStep)."""
+def reference(q, d, dims, tau, st, n, dt=1.0, phi=None):
+    """n steps in long double; phi [3][N or 1]: rotation vector of the field term (Eqs. DiscrAvr, WeqAlgo, CollisionStep, TransportStep)."""
     with q.Lattice(d, dims, tau, 1.0, dt=dt, precision="fp64") as lat:
         k = {name: np.longdouble(v) for name, v in lat.info().items()}
     nx, ny, nz = dims
@@ -56,7 +56,14 @@ def reference(q, d, dims, tau, st, n, dt=1.0):
             t = sum(v[a] * j[a] for a in range(3))
             P = (1 - k["c"] * a2 + a2 * K * sum(map(abs, v)) + 2 * K * k["alpha3"] * t +
                  4 * K * K * k["alpha4"] * t * t + K * k["alpha5"] * jj)
-            c = (W[i] + omega * (w[i] * P * rho - W[i])).reshape(4, nz, ny, nx)
+            c = W[i] + omega * (w[i] * P * rho - W[i])
+            if phi is not None:     # Rodrigues
+                th = np.sqrt((phi * phi).sum(0))
+                a = phi / th
+                s, dot = c[1:], (a * c[1:]).sum(0)
+                cross = np.stack([a[1] * s[2] - a[2] * s[1], a[2] * s[0] - a[0] * s[2], a[0] * s[1] - a[1] * s[0]])
+                c = np.concatenate([c[:1], np.cos(th) * s + np.sin(th) * cross + (1 - np.cos(th)) * dot * a])
+            c = c.reshape(4, nz, ny, nx)
             new.append(np.roll(c, (v[2], v[1], v[0]), (1, 2, 3)).reshape(4, -1))
         W = np.stack(new)
     return W
@@ -160,3 +167,42 @@ def test_density_near_a_power_of_two(q, d, dims, scale):
     E = sum(sum(map(abs, v)) * f[i] for i, v in enumerate(e)) / f.sum(0)
     assert np.max(np.abs(u - xi * np.stack(j))) < TOL
     assert np.max(np.abs(eps - 0.5 * xi * xi * (E - sum(a * a for a in j)))) < 4 * TOL
+
+
+@pytest.mark.parametrize("kind", ["uniform", "site"])
+@pytest.mark.parametrize("prec", ["fp64", "fp64df"])
+@pytest.mark.parametrize("d,dims", [(2, (19, 4, 1)), (3, (9, 4, 3))])
+def test_magnetic_field(q, d, dims, prec, kind):
+    # the rotation folded into the relaxation, and by warps that step in double
+    st = fields.random_populations(d, dims, seed=47)
+    st[:, 1] *= 1e-3                    # spin components of different size
+    N = st.shape[2]
+    B = fields.normal(7, 1, 3 * N).reshape(3, N)
+    if kind == "uniform":
+        B = B[:, :1].copy()
+    phi = 2 * np.longdouble(0.4) * B.astype(np.longdouble)
+    for n in (1, 2):
+        # for one step also a site outside the fixed-point form (its density
+        # is negative after the second)
+        st[-1, 0, 3] += 2.0 if n == 1 else -2.0
+        with q.Lattice(d, dims, 0.7, 1.0, precision=prec) as lat:
+            if kind == "site":
+                lat.set_magnetic_field_array(0.4, B)
+            else:
+                lat.set_magnetic_field(0.4, B[:, 0])
+            lat.set_state(st)
+            lat.step(n)
+            got = lat.get_state()
+        exp = reference(q, d, dims, 0.7, st, n, phi=phi)
+        # the rotation mixes the components: relative to the largest
+        assert np.max(np.abs(got - exp)) < n * TOL * np.abs(exp).max()
+
+
+def test_double_float_precision_beyond_omega_2(q):
+    # QLBM_FP64_DF is stepped by the same kernel there, in double
+    st = fields.random_populations(3, (9, 4, 3), seed=53)
+    with q.Lattice(3, (9, 4, 3), 1.0, 1.0, dt=2.5, precision="fp64df") as lat:
+        lat.set_state(st)
+        lat.step(1)
+        got = lat.get_state()
+    assert worst(got, reference(q, 3, (9, 4, 3), 1.0, st, 1, dt=2.5)) < 2 * TOL
