@@ -4,7 +4,9 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <mutex>
 #include <string>
+#include <vector>
 
 #include "internal.h"
 #include "fdparams.cuh"
@@ -49,12 +51,86 @@ int ensure_staging(qlbm_ctx *h, size_t bytes)
     return QLBM_OK;
 }
 
-// Reads and clears the device flag word (stream must be idle).
-int check_flags(qlbm_ctx *h)
+}  // namespace
+
+namespace qlbm {
+
+// What a synchronising call reads back, into host memory that the device
+// writes itself: one small kernel and one wait instead of a copy (through a
+// staging buffer, as the destination is pageable) and two waits.
+__global__ void k_report(const unsigned *flags, const unsigned long long *counter, HostReport *out)
 {
-    unsigned f = 0;
-    CK(h, cudaMemcpyAsync(&f, h->flags, sizeof(f), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
+    out->flags = *flags;
+    if (counter) out->counter = *counter;
+}
+
+}  // namespace qlbm
+
+namespace {
+
+// Report slots come from pages of 32 (allocating host memory that the device
+// can write takes ~0.1 ms, a tenth of creating a small handle).  A page goes
+// when its last slot is returned, but for one; the mutex covers handles made
+// and destroyed by several threads.
+struct ReportPage {
+    HostReport *slots;
+    unsigned used;      // bit i: slot i is taken
+};
+std::mutex report_mutex;
+std::vector<ReportPage> report_pages;
+constexpr size_t kReportSlot = 128;
+static_assert(sizeof(HostReport) <= kReportSlot, "a report fits its slot");
+HostReport *report_slot(const ReportPage &p, int i)
+{
+    return reinterpret_cast<HostReport *>(reinterpret_cast<char *>(p.slots) + kReportSlot * (size_t)i);
+}
+
+cudaError_t take_report(HostReport **host, HostReport **dev)
+{
+    std::lock_guard<std::mutex> lock(report_mutex);
+    size_t k = 0;
+    while (k < report_pages.size() && report_pages[k].used == ~0u) ++k;
+    if (k == report_pages.size()) {
+        ReportPage p{nullptr, 0u};
+        cudaError_t e = cudaHostAlloc(&p.slots, 32 * kReportSlot, cudaHostAllocMapped | cudaHostAllocPortable);
+        if (e != cudaSuccess) return e;
+        try {
+            report_pages.push_back(p);
+        } catch (...) {     // no exception crosses the ABI
+            cudaFreeHost(p.slots);
+            return cudaErrorMemoryAllocation;
+        }
+    }
+    ReportPage &p = report_pages[k];
+    int i = 0;
+    while (p.used >> i & 1u) ++i;
+    HostReport *r = report_slot(p, i);
+    cudaError_t e = cudaHostGetDevicePointer(dev, r, 0);
+    if (e != cudaSuccess) return e;
+    p.used |= 1u << i;
+    *host = r;
+    return cudaSuccess;
+}
+
+void give_report(HostReport *r)
+{
+    std::lock_guard<std::mutex> lock(report_mutex);
+    for (size_t k = 0; k < report_pages.size(); ++k)
+        for (int i = 0; i < 32; ++i)
+            if (report_slot(report_pages[k], i) == r) {
+                report_pages[k].used &= ~(1u << i);
+                if (!report_pages[k].used && report_pages.size() > 1) {
+                    cudaFreeHost(report_pages[k].slots);
+                    report_pages.erase(report_pages.begin() + (long)k);
+                }
+                return;
+            }
+}
+
+// The message and code of the flags in the handle's report; clears them.
+int report_flags(qlbm_ctx *h)
+{
+    const unsigned f = h->report->flags;
     if (f) {
         CK(h, cudaMemsetAsync(h->flags, 0, sizeof(unsigned), h->stream));
         CK(h, cudaStreamSynchronize(h->stream));
@@ -64,6 +140,16 @@ int check_flags(qlbm_ctx *h)
     if (f & FLAG_NONFINITE) return fail(h, QLBM_ERR_NONFINITE, "a step met a non-finite moment");
     if (f & FLAG_NONPOSITIVE) return fail(h, QLBM_ERR_NONPOSITIVE_DENSITY, "a step met tr rho <= 0");
     return QLBM_OK;
+}
+
+// Waits for the stream, then reads and clears the device flag word; counter:
+// a device counter to read with it (into the report).
+int check_flags(qlbm_ctx *h, const unsigned long long *counter = nullptr)
+{
+    k_report<<<1, 1, 0, h->stream>>>(h->flags, counter, h->report_dev);
+    CK(h, cudaGetLastError());
+    CK(h, cudaStreamSynchronize(h->stream));
+    return report_flags(h);
 }
 
 bool valid(qlbm_ctx *h) { return h != nullptr && h->pop != nullptr; }
@@ -184,8 +270,10 @@ int set_global_error(int code, const char *msg) { return fail(nullptr, code, msg
 
 __global__ void __launch_bounds__(kRedBlock)
 k_conserved_final(const double *__restrict__ partials, int nparts, double xi, int64_t N,
-                  double *__restrict__ out)
+                  double *__restrict__ out, const unsigned *flags, unsigned *flags_out)
 {
+    wait_for_previous();
+    if (flags_out && threadIdx.x == 0) *flags_out = *flags;
     // thread (r, i) sums component i of rows r, r + 32, ...: the double pipe
     // (64 cycles per warp instruction) is what this block waits for, so no
     // thread adds a component it does not keep (one thread per row with eight
@@ -246,9 +334,9 @@ k_field_quaternions(const double *__restrict__ B, int64_t N, double mu_dt, V *__
 
 cudaError_t launch_conserved_final(qlbm_ctx *h)
 {
-    k_conserved_final<<<1, kRedBlock, 0, h->stream>>>(h->partials, h->red_grid ? h->red_grid : h->nred, h->hc.xi,
-                                                      h->g.N, h->red_out);
-    return cudaGetLastError();
+    return launch_chained(k_conserved_final, dim3(1), dim3(kRedBlock), 0, h->stream, h->partials,
+                          h->red_grid ? h->red_grid : h->nred, h->hc.xi, h->g.N, h->report_dev->sums, h->flags,
+                          &h->report_dev->flags);
 }
 
 }  // namespace qlbm
@@ -313,6 +401,7 @@ int qlbm_create(qlbm_handle *out, int lattice, const int64_t dims[3], double tau
     h->nred = (int)(nred < 1024 ? nred : 1024);
     if (e == cudaSuccess) e = cudaMalloc(&h->partials, (size_t)h->nred * 8 * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&h->red_out, 8 * sizeof(double));
+    if (e == cudaSuccess) e = take_report(&h->report, &h->report_dev);
     if (e != cudaSuccess) {
         char buf[256];
         snprintf(buf, sizeof(buf), "qlbm_create: %s (population buffer %zu bytes)",
@@ -333,6 +422,7 @@ void qlbm_destroy(qlbm_handle h)
     if (h->flags) cudaFree(h->flags);
     if (h->partials) cudaFree(h->partials);
     if (h->red_out) cudaFree(h->red_out);
+    if (h->report) give_report(h->report);
     if (h->staging) cudaFree(h->staging);
     for (int i = 0; i < 2; ++i)
         if (h->lam[i]) cudaFree(h->lam[i]);
@@ -426,7 +516,6 @@ int64_t qlbm_time(qlbm_handle h) { return h ? h->t : -1; }
 int qlbm_sync(qlbm_handle h)
 {
     if (!valid(h)) return fail(h, QLBM_ERR_INVALID_ARG, "qlbm_sync: bad handle");
-    CK(h, cudaStreamSynchronize(h->stream));
     return check_flags(h);
 }
 
@@ -447,7 +536,6 @@ int qlbm_moments(qlbm_handle h, double *rho4, double *u, double *eps, int ptr_ki
     } else {
         CK(h, h->ops->moments(h, rho4, u, eps));
     }
-    CK(h, cudaStreamSynchronize(h->stream));
     return check_flags(h);
 }
 
@@ -456,9 +544,9 @@ int qlbm_conserved(qlbm_handle h, double *out)
     if (!valid(h) || !out) return fail(h, QLBM_ERR_INVALID_ARG, "qlbm_conserved: bad argument");
     CK(h, h->ops->conserved_partial(h));
     CK(h, launch_conserved_final(h));
-    CK(h, cudaMemcpyAsync(out, h->red_out, 8 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
-    return check_flags(h);
+    memcpy(out, h->report->sums, sizeof(h->report->sums));
+    return report_flags(h);
 }
 
 int qlbm_get_state(qlbm_handle h, double *buf, int ptr_kind)
@@ -475,7 +563,6 @@ int qlbm_get_state(qlbm_handle h, double *buf, int ptr_kind)
     } else {
         CK(h, h->ops->get_state(h, buf));
     }
-    CK(h, cudaStreamSynchronize(h->stream));
     return check_flags(h);
 }
 
@@ -524,7 +611,6 @@ int qlbm_save_checkpoint(qlbm_handle h, void *buf, int ptr_kind)
     for (int64_t p = 0; p < image_planes(h); ++p)
         CK(h, cudaMemcpyAsync(static_cast<char *>(buf) + p * row, reinterpret_cast<char *>(h->staging) + p * pitch,
                               row, kind, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
     return check_flags(h);
 }
 
@@ -789,7 +875,6 @@ int qlbm_set_magnetic_field_array(qlbm_handle h, double mu, const double *B, int
     }
     // earlier steps' flags are reported first, so that a bad field is not
     // mistaken for them
-    CK(h, cudaStreamSynchronize(h->stream));
     int rc = check_flags(h);
     if (rc) return rc;
     const unsigned nb = (unsigned)((N + 255) / 256);
@@ -798,7 +883,6 @@ int qlbm_set_magnetic_field_array(qlbm_handle h, double mu, const double *B, int
     else
         k_field_quaternions<<<nb, 256, 0, h->stream>>>(src, N, mu * h->dt, static_cast<float4 *>(h->qfield), h->flags);
     CK(h, cudaGetLastError());
-    CK(h, cudaStreamSynchronize(h->stream));
     if (check_flags(h) != QLBM_OK) {
         h->mag = FIELD_NONE;
         return fail(h, QLBM_ERR_INVALID_ARG, "qlbm_set_magnetic_field_array: non-finite field value (field switched off)");
@@ -845,11 +929,9 @@ int qlbm_fd_params(qlbm_handle h, double *beta, double *mu_up, double *mu_dn, do
     } else {
         CK(h, h->ops->fd_params(h, beta, mu_up, mu_dn, axis));
     }
-    unsigned long long nf = 0;
-    CK(h, cudaMemcpyAsync(&nf, h->fd_fail, sizeof(nf), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
-    if (nfail) *nfail = (int64_t)nf;
-    return check_flags(h);
+    const int rc = check_flags(h, h->fd_fail);
+    if (nfail) *nfail = (int64_t)h->report->counter;
+    return rc;
 }
 
 int qlbm_step_fd_output(qlbm_handle h, float *beta, float *mu_up, float *mu_dn, float *axis, int64_t *nfail,
@@ -886,11 +968,9 @@ int qlbm_step_fd_output(qlbm_handle h, float *beta, float *mu_up, float *mu_dn, 
         CK(h, cudaMemcpyAsync(axis, ax, 3 * N * sizeof(float), cudaMemcpyDeviceToHost, h->stream));
     }
     if (count || ptr_kind == QLBM_HOST) {
-        unsigned long long nf = 0;
-        if (count) CK(h, cudaMemcpyAsync(&nf, h->fd_fail, sizeof(nf), cudaMemcpyDeviceToHost, h->stream));
-        CK(h, cudaStreamSynchronize(h->stream));
-        if (count) *nfail = (int64_t)nf;
-        return check_flags(h);
+        const int rc = check_flags(h, count ? h->fd_fail : nullptr);
+        if (count) *nfail = (int64_t)h->report->counter;
+        return rc;
     }
     return QLBM_OK;
 }
@@ -911,11 +991,9 @@ int qlbm_negative_eq_count(qlbm_handle h, int64_t *count, uint32_t *mask, int pt
     CK(h, h->ops->negative_eq(h, h->neg_count, m));
     if (mask && ptr_kind == QLBM_HOST)
         CK(h, cudaMemcpyAsync(mask, m, N * sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
-    unsigned long long c = 0;
-    CK(h, cudaMemcpyAsync(&c, h->neg_count, sizeof(c), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
-    *count = (int64_t)c;
-    return check_flags(h);
+    const int rc = check_flags(h, h->neg_count);
+    *count = (int64_t)h->report->counter;
+    return rc;
 }
 
 int qlbm_fd_params_adjoint(qlbm_handle h, const double *g_beta, const double *g_mu_up, const double *g_mu_dn,
@@ -925,7 +1003,6 @@ int qlbm_fd_params_adjoint(qlbm_handle h, const double *g_beta, const double *g_
     if (ptr_kind != QLBM_HOST && ptr_kind != QLBM_DEVICE) return fail(h, QLBM_ERR_INVALID_ARG, "bad ptr_kind");
     if (ptr_kind == QLBM_DEVICE) {
         CK(h, h->ops->fd_params_adjoint(h, g_beta, g_mu_up, g_mu_dn, g_axis, lam));
-        CK(h, cudaStreamSynchronize(h->stream));
         return check_flags(h);
     }
     const size_t N = (size_t)h->g.N, ld = (size_t)h->b * 4 * N;
@@ -939,7 +1016,6 @@ int qlbm_fd_params_adjoint(qlbm_handle h, const double *g_beta, const double *g_
     CK(h, h->ops->fd_params_adjoint(h, g_beta ? gb : nullptr, g_mu_up ? gu : nullptr, g_mu_dn ? gd : nullptr,
                                     g_axis ? ga : nullptr, l));
     CK(h, cudaMemcpyAsync(lam, l, ld * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    CK(h, cudaStreamSynchronize(h->stream));
     return check_flags(h);
 }
 

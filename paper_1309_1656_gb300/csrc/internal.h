@@ -28,6 +28,13 @@ int compute_constants(int d, double beta0, HostConsts *out);
 
 struct LatticeOps;
 
+// What a synchronising call reads back (host memory mapped into the device).
+struct HostReport {
+    double sums[8];                 // qlbm_conserved
+    unsigned long long counter;     // unresolved sites, flagged pairs
+    unsigned flags;
+};
+
 }  // namespace qlbm
 
 struct qlbm_ctx {
@@ -45,6 +52,7 @@ struct qlbm_ctx {
     unsigned *flags = nullptr;      // device flag word
     double *partials = nullptr;     // device reduction scratch [nred][8]
     double *red_out = nullptr;      // device [8]
+    qlbm::HostReport *report = nullptr, *report_dev = nullptr;   // the same memory, host and device address
     int nred = 0;                   // rows of partials (the most blocks a reduction launches)
     int red_grid = 0;               // blocks of the reduction: whole waves of resident blocks, <= nred
     double *staging = nullptr;      // device staging for host inputs/outputs

@@ -131,6 +131,7 @@ k_conserved_partial_df(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g
     using R = typename Codec::R;
     constexpr int Q = Lattice<D>::Q;
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    wait_for_previous();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     df tot[8];
 #pragma unroll
@@ -162,6 +163,7 @@ k_conserved_partial_df(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g
 #pragma unroll
         for (int k = 0; k < 8; ++k) tot[k] = tot[k] + a[k].value();
     }
+    let_next_start();
     // warp sum in double-float, then one conversion per warp
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
@@ -192,9 +194,10 @@ k_conserved_partial_df(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g
 }
 
 // Sums nparts rows of 8 partials in a fixed order; out[0..7] then scaled:
-// density /N, momentum xi/N, energy xi^2/(2N).
+// density /N, momentum xi/N, energy xi^2/(2N).  *flags_out (if not NULL)
+// receives *flags.
 __global__ void __launch_bounds__(kRedBlock)
 k_conserved_final(const double *__restrict__ partials, int nparts, double xi, int64_t N,
-                  double *__restrict__ out);
+                  double *__restrict__ out, const unsigned *flags, unsigned *flags_out);
 
 }  // namespace qlbm

@@ -196,16 +196,16 @@ template <int D, class Codec> struct Launchers {
             if (!grid)
                 return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
                     resident, k_conserved_partial_df<D, Codec, SWAPPED>, kRedBlock, 0);
-            k_conserved_partial_df<D, Codec, SWAPPED><<<grid, kRedBlock, 0, h->stream>>>(
-                planes(h), h->g, make_codec<Codec>(h), h->partials);
+            return launch_chained(k_conserved_partial_df<D, Codec, SWAPPED>, dim3((unsigned)grid), dim3(kRedBlock), 0, h->stream,
+                                  planes(h), h->g, make_codec<Codec>(h), h->partials);
         } else {
             if (!grid)
                 return cudaOccupancyMaxActiveBlocksPerMultiprocessor(resident, k_conserved_partial<D, Codec, SWAPPED>,
                                                                      kRedBlock, 0);
-            k_conserved_partial<D, Codec, SWAPPED><<<grid, kRedBlock, 0, h->stream>>>(
-                planes(h), h->g, make_codec<Codec>(h), make_chunks(h->g), make_quad_ref(h->hc), h->partials);
+            return launch_chained(k_conserved_partial<D, Codec, SWAPPED>, dim3((unsigned)grid), dim3(kRedBlock), 0, h->stream,
+                                  planes(h), h->g, make_codec<Codec>(h), make_chunks(h->g), make_quad_ref(h->hc),
+                                  h->partials);
         }
-        return cudaGetLastError();
     }
 
     static cudaError_t conserved_partial(qlbm_ctx *h)

@@ -119,7 +119,7 @@ extern "C" int qlbm_conserved_static(int lattice, const int64_t dims[3], double 
         k_conserved_partial_canonical<3><<<nblocks, kRedBlock, 0, st>>>(state, N, partials);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {
-        k_conserved_final<<<1, kRedBlock, 0, st>>>(partials, nblocks, hc.xi, N, out);
+        k_conserved_final<<<1, kRedBlock, 0, st>>>(partials, nblocks, hc.xi, N, out, nullptr, nullptr);
         e = cudaGetLastError();
     }
     if (e != cudaSuccess)

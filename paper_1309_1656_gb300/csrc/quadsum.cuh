@@ -462,6 +462,7 @@ k_conserved_partial(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, C
     const unsigned all = 0xffffffffu;
     const int c = threadIdx.x & 3, nw = (int)gridDim.x * (kRedBlock / 32);
     double acc[2] = {0.0, 0.0};
+    wait_for_previous();
     for (int chunk = (int)((blockIdx.x * kRedBlock + threadIdx.x) >> 5); chunk < ch.total; chunk += nw) {
         SiteIdx si;
         const bool active = quad_site(g, ch, chunk, si);
@@ -491,6 +492,7 @@ k_conserved_partial(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, C
             acc[1] += v;
         }
     }
+    let_next_start();
     if (D == 2 && c == 3) acc[1] = 0.0;
     // over the warp's eight sites, then over the block's warps
     __shared__ double sh[kRedBlock / 32][8];
