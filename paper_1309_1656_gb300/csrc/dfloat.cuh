@@ -310,8 +310,12 @@ struct CodecDF {
         p[0] = make_float4(f.hi, x.hi, y.hi, z.hi);
         p[lo] = make_float4(f.lo, x.lo, y.lo, z.lo);
     }
-    __device__ __forceinline__ double to_double(R v, int, int) const { return v.to_double(); }
-    __device__ __forceinline__ S from_double(double v, int, int) const { return df(v); }
+    __device__ __forceinline__ double to_double(R v, int, int) const { return widen(v.hi) + widen(v.lo); }
+    __device__ __forceinline__ S from_double(double v, int, int) const
+    {
+        const float h = narrow(v);
+        return df(h, narrow(v - widen(h)));
+    }
 };
 
 }  // namespace qlbm
