@@ -22,6 +22,8 @@
 // arithmetic and are not differentiated.
 #pragma once
 
+#include <utility>
+
 #include "kernels.cuh"
 
 namespace qlbm {
@@ -143,66 +145,37 @@ __device__ __forceinline__ void unrotate(R &mx, R &my, R &mz, const R (&rot)[9])
     mz = rot[2] * x + rot[5] * y + rot[8] * z;
 }
 
-template <int D, class Codec, int q, int FIELD>
-__device__ __forceinline__ void adj_accumulate(const Planes<typename Codec::S, Lattice<D>::Q> &st,
-                                               const Planes<typename Codec::R, Lattice<D>::Q> &lin,
-                                               const Grid &g, const SiteIdx &si, const Codec &codec,
-                                               const Coll<typename Codec::R> &k,
-                                               const typename Codec::R (&rot)[9], typename Codec::R (&fw)[8],
-                                               typename Codec::R &dot, MuMom<typename Codec::R> &A,
-                                               MuMom<typename Codec::R> &Bx, MuMom<typename Codec::R> &By,
-                                               MuMom<typename Codec::R> &Bz)
+// f(std::integral_constant<int, q>) for every direction.
+template <class F, int... q> __device__ __forceinline__ void for_directions(F &&f, std::integer_sequence<int, q...>)
 {
-    using R = typename Codec::R;
-    R f, sx, sy, sz;
-    codec.load4(st.p[q] + si.s, f, sx, sy, sz);
-    const int s = neighbour(g, si, cx<D>(q), cy<D>(q), cz<D>(q));
-    R mf, mx, my, mz;
-    ldq(lin.p[q] + s, mf, mx, my, mz);
-    if constexpr (FIELD != FIELD_NONE) unrotate(mx, my, mz, rot);
-    fw[0] += f;
-    fw[1] += sx;
-    fw[2] += sy;
-    fw[3] += sz;
-    if (cx<D>(q)) fw[4] += cx<D>(q) * f;
-    if (cy<D>(q)) fw[5] += cy<D>(q) * f;
-    if (cz<D>(q)) fw[6] += cz<D>(q) * f;
-    if (cnorm2<D>(q)) fw[7] += cnorm2<D>(q) * f;
-    dot += mf * f + mx * sx + my * sy + mz * sz;
-    const R w = k.w[cnorm2<D>(q)];
-    A.template add<D, q>(w * mf);
-    Bx.template add<D, q>(w * mx);
-    By.template add<D, q>(w * my);
-    Bz.template add<D, q>(w * mz);
+    (f(std::integral_constant<int, q>{}), ...);
 }
 
-template <int D, class Codec, int q, int FIELD>
-struct AdjLoop {
-    static __device__ __forceinline__ void run(const Planes<typename Codec::S, Lattice<D>::Q> &st,
-                                               const Planes<typename Codec::R, Lattice<D>::Q> &lin,
-                                               const Grid &g, const SiteIdx &si, const Codec &codec,
-                                               const Coll<typename Codec::R> &k,
-                                               const typename Codec::R (&rot)[9], typename Codec::R (&fw)[8],
-                                               typename Codec::R &dot, MuMom<typename Codec::R> &A,
-                                               MuMom<typename Codec::R> &Bx, MuMom<typename Codec::R> &By,
-                                               MuMom<typename Codec::R> &Bz)
-    {
-        adj_accumulate<D, Codec, q, FIELD>(st, lin, g, si, codec, k, rot, fw, dot, A, Bx, By, Bz);
-        AdjLoop<D, Codec, q + 1, FIELD>::run(st, lin, g, si, codec, k, rot, fw, dot, A, Bx, By, Bz);
-    }
+// D3Q19 with cotangents in single precision: W^n and mu pass through shared
+// memory, all 38 copies of a site started (cp.async) before the first is
+// waited for, and the second pass finds mu there.  Loaded into registers as
+// the accumulators left room for, they kept too few bytes in flight
+// (long-scoreboard stall 11.7 per issue): 96^3 FP32 146.6 -> 135.9 us per
+// reverse step, 128^3 319.8 -> 288.8 (FP16 286.5 -> 254.3), 33 x 35 x 40 16.3 ->
+// 12.3.  D2Q9's 18 loads all fit in registers (1024^2 81.0, staged 90.9); in
+// double a site's vectors would leave room for 4 warps per SM.
+template <int D, class Codec> struct AdjStaged {
+    static constexpr bool value = D == 3 && sizeof(typename Codec::R) == 4;
 };
-template <int D, class Codec, int FIELD> struct AdjLoop<D, Codec, Lattice<D>::Q, FIELD> {
-    static __device__ __forceinline__ void run(const Planes<typename Codec::S, Lattice<D>::Q> &,
-                                               const Planes<typename Codec::R, Lattice<D>::Q> &,
-                                               const Grid &, const SiteIdx &, const Codec &,
-                                               const Coll<typename Codec::R> &,
-                                               const typename Codec::R (&)[9], typename Codec::R (&)[8],
-                                               typename Codec::R &, MuMom<typename Codec::R> &,
-                                               MuMom<typename Codec::R> &, MuMom<typename Codec::R> &,
-                                               MuMom<typename Codec::R> &)
-    {
-    }
-};
+template <int D, class Codec> constexpr size_t adj_smem_bytes(int block)
+{
+    return AdjStaged<D, Codec>::value ? (size_t)Lattice<D>::Q * block *
+                                         (sizeof(typename QuadOf<typename Codec::S>::V) + sizeof(typename QuadOf<typename Codec::R>::V))
+                                   : 0;
+}
+__device__ __forceinline__ void adj_decode(const CodecF32 &, const float4 *p, float &f, float &x, float &y, float &z)
+{
+    ldq(p, f, x, y, z);
+}
+__device__ __forceinline__ void adj_decode(const CodecF16Dev &c, const uint2 *p, float &f, float &x, float &y, float &z)
+{
+    c.decode4(*p, f, x, y, z);
+}
 
 // One reverse step.  state: W^n in natural order; lam_in: lambda^{n+1};
 // lam_out: lambda^n (natural order, arithmetic type R).  dtau_acc[block] +=
@@ -213,18 +186,25 @@ template <int D, class Codec, int FIELD> struct AdjLoop<D, Codec, Lattice<D>::Q,
 // cotangent moments sum_k w_k mu_k (1, i_k, |i_k|^2, i_k i_k^T).  Every
 // per-direction sum of the transpose above is a polynomial of degree <= 2 in
 // i_k times w_k mu_k, so these moments give them once the forward moments
-// are known.  Pass 2 re-reads mu (cache hits; the index carries the
-// run-time zero so the compiler does not keep pass 1's values live) and
-// writes lambda^n.
+// are known.  Pass 2 re-reads mu (shared memory, or cache hits; the index
+// carries the run-time zero so the compiler does not keep pass 1's values
+// live) and writes lambda^n.
 template <int D, class Codec, int FIELD>
-__global__ void __launch_bounds__(kAdjBlock, Codec::MIN_BLOCKS)
+__global__ void __launch_bounds__(kAdjBlock, AdjStaged<D, Codec>::value ? 2 : Codec::MIN_BLOCKS)
 k_adjoint(const Planes<typename Codec::S, Lattice<D>::Q> st, const Planes<typename Codec::R, Lattice<D>::Q> lin,
           const Planes<typename Codec::R, Lattice<D>::Q> lout, Grid g, Coll<typename Codec::R> k,
           Codec codec, double *__restrict__ dtau_acc)
 {
     using R = typename Codec::R;
+    using VS = typename QuadOf<typename Codec::S>::V;
+    using VR = typename QuadOf<R>::V;
     constexpr int Q = Lattice<D>::Q;
-    constexpr bool DEV = Codec::DEV;
+    constexpr bool DEV = Codec::DEV, STAGED = AdjStaged<D, Codec>::value;
+    // vector q of this thread at mu_st[q * bw] and w_st[q * bw]
+    extern __shared__ __align__(16) unsigned char adj_smem[];
+    const int bw = blockDim.x;
+    VR *const mu_st = reinterpret_cast<VR *>(adj_smem) + threadIdx.x;
+    VS *const w_st = reinterpret_cast<VS *>(reinterpret_cast<VR *>(adj_smem) + Q * bw) + threadIdx.x;
     SiteIdx si;
     wait_for_previous();
     const bool active = site_of_block(g, si);
@@ -241,7 +221,44 @@ k_adjoint(const Planes<typename Codec::S, Lattice<D>::Q> st, const Planes<typena
         // the spins collided here; their cotangents take its transpose)
         R rot[9];
         if constexpr (FIELD != FIELD_NONE) field_rotation<FIELD>(k, si.s, rot);
-        AdjLoop<D, Codec, 0, FIELD>::run(st, lin, g, si, codec, k, rot, fw, dot, A, Bx, By, Bz);
+        if constexpr (STAGED) {
+            const NbOff nb = nb_offsets(g, si);
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                cp_async_vec<sizeof(VS)>(w_st + q * bw, st.p[q] + si.s);
+                cp_async_vec<sizeof(VR)>(mu_st + q * bw, lin.p[q] + nb_at(nb, si.s, cx<D>(q), cy<D>(q), cz<D>(q)));
+            }
+            cp_async_commit();
+            cp_async_wait<0>();
+        }
+        for_directions(
+            [&](auto qc) {
+                constexpr int q = decltype(qc)::value;
+                R f, sx, sy, sz, mf, mx, my, mz;
+                if constexpr (STAGED) {
+                    adj_decode(codec, w_st + q * bw, f, sx, sy, sz);
+                    ldq(mu_st + q * bw, mf, mx, my, mz);
+                } else {
+                    codec.load4(st.p[q] + si.s, f, sx, sy, sz);
+                    ldq(lin.p[q] + neighbour(g, si, cx<D>(q), cy<D>(q), cz<D>(q)), mf, mx, my, mz);
+                }
+                if constexpr (FIELD != FIELD_NONE) unrotate(mx, my, mz, rot);
+                fw[0] += f;
+                fw[1] += sx;
+                fw[2] += sy;
+                fw[3] += sz;
+                if (cx<D>(q)) fw[4] += cx<D>(q) * f;
+                if (cy<D>(q)) fw[5] += cy<D>(q) * f;
+                if (cz<D>(q)) fw[6] += cz<D>(q) * f;
+                if (cnorm2<D>(q)) fw[7] += cnorm2<D>(q) * f;
+                dot += mf * f + mx * sx + my * sy + mz * sz;
+                const R w = k.w[cnorm2<D>(q)];
+                A.template add<D, q>(w * mf);
+                Bx.template add<D, q>(w * mx);
+                By.template add<D, q>(w * my);
+                Bz.template add<D, q>(w * mz);
+            },
+            std::make_integer_sequence<int, Q>{});
         // forward moments
         const R dn = DEV ? fw[0] : fw[0] - R(1);
         const R n = DEV ? R(1) + fw[0] : fw[0];
@@ -302,9 +319,9 @@ k_adjoint(const Planes<typename Codec::S, Lattice<D>::Q> st, const Planes<typena
         let_next_start();
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
-            const int s = neighbour(g, s2, cx<D>(q), cy<D>(q), cz<D>(q));
             R mf, mx, my, mz;
-            ldq(lin.p[q] + s, mf, mx, my, mz);
+            if constexpr (STAGED) ldq(mu_st + q * bw + g.zero, mf, mx, my, mz);
+            else ldq(lin.p[q] + neighbour(g, s2, cx<D>(q), cy<D>(q), cz<D>(q)), mf, mx, my, mz);
             if constexpr (FIELD != FIELD_NONE) unrotate(mx, my, mz, rot);
             stq(lout.p[q] + s2.s,
                 omc * mf + nbar + (cx<D>(q) * Jbx2 + cy<D>(q) * Jby2 + cz<D>(q) * Jbz2) + cnorm2<D>(q) * Eb,
@@ -395,42 +412,85 @@ k_lam_export(const Planes<R, Lattice<D>::Q> lam, Grid g, double *__restrict__ ou
 
 // Adjoint of the equilibrium initialisation W_i = w_i P_i(u, eps) rho
 // (Eq. WeqAlgo with given u and eps): gradients with respect to rho4
-// (n, S), u and eps, in double.
+// (n, S), u and eps, in double.  Bound by the double pipe (64 cycles per warp
+// instruction): the cotangents of P_i are summed to moments by pairs and
+// classes, the gradients of u and eps formed from those once, and P_i shares
+// its even and odd part within a pair, ~305 instructions at D3Q19 instead of
+// ~565: 96^3 861 -> 490 us.  rxi: 1 / xi.
 template <int D>
 __global__ void __launch_bounds__(kStepBlock)
-k_init_adjoint(const double *__restrict__ lam, Grid g, InitConsts ic, const double *__restrict__ rho4,
-               const double *__restrict__ u, const double *__restrict__ eps, double *__restrict__ grho4,
-               double *__restrict__ gu, double *__restrict__ geps)
+k_init_adjoint(const double *__restrict__ lam, Grid g, InitConsts ic, double rxi,
+               const double *__restrict__ rho4, const double *__restrict__ u, const double *__restrict__ eps,
+               double *__restrict__ grho4, double *__restrict__ gu, double *__restrict__ geps)
 {
     constexpr int Q = Lattice<D>::Q;
     SiteIdx si;
     if (!site_of_block(g, si)) return;
     const int64_t N = g.N, s = si.s;
     const double n = rho4[s], Sx = rho4[N + s], Sy = rho4[2 * N + s], Sz = rho4[3 * N + s];
-    const double jx = u[s] / ic.xi, jy = u[N + s] / ic.xi, jz = (D == 3) ? u[2 * N + s] / ic.xi : 0.0;
-    const double e = eps ? eps[s] : ic.eps0;
-    const double be = ic.beta0 * e;
-    double gn = 0, gx = 0, gy = 0, gz = 0, gjx = 0, gjy = 0, gjz = 0, gbe = 0;
+    const double j[3] = {u[s] * rxi, u[N + s] * rxi, D == 3 ? u[2 * N + s] * rxi : 0.0};
+    const double be = ic.beta0 * (eps ? eps[s] : ic.eps0);
+    // P_i = a_cls + c3 t + c4 t^2, t = i.j
+    const double a2 = (be - ic.c) * ic.inv_mc2;
+    const double a0 = 1.0 - ic.c * a2 + ic.c5 * (j[0] * j[0] + j[1] * j[1] + j[2] * j[2]);
+    double gn = 0, gx = 0, gy = 0, gz = 0;
+    // n lam_f + S . lam_s of direction q (the cotangent of P_q but for w), with
+    // the direction's share of the gradient of rho4
+    auto take = [&](int q, double wP) {
+        const double *v = lam + (int64_t)(4 * q) * N + s;
+        const double lf = v[0], lx = v[N], ly = v[2 * N], lz = v[3 * N];
+        gn += wP * lf;
+        gx += wP * lx;
+        gy += wP * ly;
+        gz += wP * lz;
+        return n * lf + Sx * lx + Sy * ly + Sz * lz;
+    };
+    // moments of the cotangents of P: sum, first, second by axis and mixed
+    const double w1 = ic.w[1], w2 = ic.w[2];
+    double m0 = ic.w[0] * take(Q / 2, ic.w[0] * a0), m1[3] = {0.0, 0.0, 0.0}, mm[3] = {0.0, 0.0, 0.0}, mixed[3];
+    const double b1 = w1 * (a0 + a2 * ic.K);
 #pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        const int cls = cnorm2<D>(q);
-        const double w = ic.w[cls];
-        const double P = poly_P_d<D>(ic, q, jx, jy, jz, be);
-        const double lf = lam[(int64_t)(4 * q) * N + s], lx = lam[(int64_t)(4 * q + 1) * N + s],
-                     ly = lam[(int64_t)(4 * q + 2) * N + s], lz = lam[(int64_t)(4 * q + 3) * N + s];
-        gn += w * P * lf;
-        gx += w * P * lx;
-        gy += w * P * ly;
-        gz += w * P * lz;
-        const double Pb = w * (n * lf + Sx * lx + Sy * ly + Sz * lz);   // cotangent of P_q
-        const double t = cx<D>(q) * jx + cy<D>(q) * jy + cz<D>(q) * jz;
-        const double dPdt = ic.c3 + 2.0 * ic.c4 * t;
-        gjx += Pb * (dPdt * cx<D>(q) + 2.0 * ic.c5 * jx);
-        gjy += Pb * (dPdt * cy<D>(q) + 2.0 * ic.c5 * jy);
-        gjz += Pb * (dPdt * cz<D>(q) + 2.0 * ic.c5 * jz);
-        // P = alpha1 + alpha2 K|i|^2 + ..., alpha2 = (be - c)/(m - c^2), alpha1 = 1 - c alpha2
-        gbe += Pb * ic.inv_mc2 * (ic.K * cls - ic.c);
+    for (int a = 0; a < D; ++a) {
+        const int q = direction_of<D>(a == 0, a == 1, a == 2);
+        const double e = b1 + (w1 * ic.c4) * (j[a] * j[a]), o = (w1 * ic.c3) * j[a];
+        const double p = take(q, e + o), m = take(Q - 1 - q, e - o);
+        mm[a] = w1 * (p + m);
+        m1[a] = w1 * (p - m);
+        m0 += mm[a];
     }
+    const double b2 = w2 * (a0 + a2 * (2.0 * ic.K));
+#pragma unroll
+    for (int a = 0; a < D - 1; ++a)
+#pragma unroll
+        for (int b = a + 1; b < D; ++b) {
+            const double ts = j[a] + j[b], td = j[a] - j[b];
+            const int qs = direction_of<D>(a == 0, a == 1 || b == 1, b == 2);
+            const int qd = direction_of<D>(a == 0, a == 1 ? 1 : (b == 1 ? -1 : 0), b == 2 ? -1 : 0);
+            const double es = b2 + (w2 * ic.c4) * (ts * ts), os = (w2 * ic.c3) * ts;
+            const double ed = b2 + (w2 * ic.c4) * (td * td), od = (w2 * ic.c3) * td;
+            const double p = take(qs, es + os), m = take(Q - 1 - qs, es - os);
+            const double r = take(qd, ed + od), l = take(Q - 1 - qd, ed - od);
+            const double pm = p + m, rl = r + l, dp = p - m, dr = r - l, all = w2 * (pm + rl);
+            m0 += all;
+            mm[a] += all;
+            mm[b] += all;
+            mixed[a + b - 1] = w2 * (pm - rl);
+            m1[a] += w2 * (dp + dr);
+            m1[b] += w2 * (dp - dr);
+        }
+    // d P_i / d j = (c3 + 2 c4 i.j) i + 2 c5 j;  d P_i / d be = inv_mc2 (K |i|^2 - c)
+    double gj[3];
+#pragma unroll
+    for (int a = 0; a < D; ++a) {
+        double t = mm[a] * j[a];
+#pragma unroll
+        for (int b = 0; b < D; ++b)
+            if (b != a) t += mixed[a + b - 1] * j[b];
+        gj[a] = ic.c3 * m1[a] + 2.0 * (ic.c4 * t + ic.c5 * (m0 * j[a]));
+    }
+    double m2 = mm[0] + mm[1];
+    if (D == 3) m2 += mm[2];
+    const double gbe = ic.inv_mc2 * (ic.K * m2 - ic.c * m0);
     if (grho4) {
         grho4[s] = gn;
         grho4[N + s] = gx;
@@ -438,9 +498,8 @@ k_init_adjoint(const double *__restrict__ lam, Grid g, InitConsts ic, const doub
         grho4[3 * N + s] = gz;
     }
     if (gu) {
-        gu[s] = gjx / ic.xi;
-        gu[N + s] = gjy / ic.xi;
-        if (D == 3) gu[2 * N + s] = gjz / ic.xi;
+#pragma unroll
+        for (int a = 0; a < D; ++a) gu[a * N + s] = gj[a] * rxi;
     }
     if (geps) geps[s] = gbe * ic.beta0;
 }

@@ -229,7 +229,13 @@ template <int D, class Codec> struct Launchers {
         const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
         return with_field(h->mag, [&](auto fc) {
             constexpr int F = decltype(fc)::value;
-            return launch_chained(k_adjoint<D, Codec, F>, grd, blk, 0, h->stream, planes_of<S>(h, state),
+            const size_t sm = adj_smem_bytes<D, Codec>((int)blk.x);
+            if (sm > 48u << 10) {
+                const cudaError_t e = cudaFuncSetAttribute(k_adjoint<D, Codec, F>,
+                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+                if (e != cudaSuccess) return e;
+            }
+            return launch_chained(k_adjoint<D, Codec, F>, grd, blk, sm, h->stream, planes_of<S>(h, state),
                                   planes_of<R>(h, lam_in), planes_of<R>(h, lam_out), h->g, make_coll<R>(h),
                                   make_codec<Codec>(h), h->dtau_acc);
         });
@@ -280,7 +286,8 @@ template <int D, class Codec> struct Launchers {
                                     const double *eps, double *grho4, double *gu, double *geps)
     {
         const dim3 blk = site_block(h->g), grd = site_grid(h->g, blk.x);
-        k_init_adjoint<D><<<grd, blk, 0, h->stream>>>(lam, h->g, make_init(h), rho4, u, eps, grho4, gu, geps);
+        k_init_adjoint<D><<<grd, blk, 0, h->stream>>>(lam, h->g, make_init(h), 1.0 / h->hc.xi, rho4, u, eps, grho4, gu,
+                                                      geps);
         return cudaGetLastError();
     }
 
