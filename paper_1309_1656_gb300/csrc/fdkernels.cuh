@@ -55,7 +55,7 @@ __device__ __forceinline__ void fd_solve_and_store(double n, double Sx, double S
 // Fermi-Dirac parameters of the current state, 64-bit storage.  The site sums
 // come from four lanes per site (quadsum.cuh), four chunks of eight sites per
 // warp; they pass through shared memory so that the solve has one lane per
-// site.  D3Q19 90 x 101 x 75 FP64: 2463 -> 531 us (sums in double and a solve of
+// site.  D3Q19 90 x 101 x 75 FP64: 2463 -> 267 us (sums in double and a solve of
 // three double evaluations before).
 constexpr int kFdBlock = 128;
 template <int D, class Codec, bool SWAPPED>
@@ -102,10 +102,10 @@ k_fd_params(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Codec cod
     for (int k = 0; k < 4; ++k) {
         const long long m = sh_m[warp][k][lane];
         const int u = sh_u[warp][k][lane];
-        M[k] = u == kDone ? __longlong_as_double(m) : quad_double(m, u);
+        M[k] = u == kDone ? __longlong_as_double(m) : fx_to_double_int(m, u);
     }
     const long long e = sh_m[warp][4][lane];
-    const double eps = sh_u[warp][0][lane] == kDone ? __longlong_as_double(e) : (double)(e << 2) * sc.e62;
+    const double eps = sh_u[warp][0][lane] == kDone ? __longlong_as_double(e) : fx_to_double_int(e, 2) * sc.e62;
     fd_solve_and_store<D>(M[0], M[1], M[2], M[3], eps, g.N, (int64_t)row * g.nx + x, out);
 }
 

@@ -434,13 +434,31 @@ __device__ FdParams fd_params_nested(double n, double Sx, double Sy, double Sz, 
     return p;
 }
 
-// 1/x for x within single precision's range: the float reciprocal and two
-// Newton steps.
+// v > 0 with an exponent within +-E of 1's, tested on the integer pipe.
+template <int E> __device__ __forceinline__ bool fd_within(double v)
+{
+    return (unsigned)(__double2hiint(v) - ((1023 - E) << 20)) < (unsigned)((2 * E) << 20);
+}
+
+// 1/x for x within single precision's range: from the approximate float
+// reciprocal's relative error e (~2^-23) r (1 + e + e^2).
 __device__ __forceinline__ double fd_recip(double x)
 {
-    double r = (double)(1.0f / (float)x);
-    r = fma(r, fma(-x, r, 1.0), r);
-    return fma(r, fma(-x, r, 1.0), r);
+    const double r = widen(__fdividef(1.0f, narrow(x))), e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// sqrt(q) and, to ~2^-43, 0.5 / sqrt(q), q within single precision's range:
+// the float reciprocal root, one coupled Newton step for both and a residual
+// correction of the root.
+__device__ __forceinline__ double fd_sqrt(double q, double &half_r)
+{
+    const float y = rsqrtf(narrow(q));
+    double s = q * widen(y), h = widen(0.5f * y);
+    const double e = fma(-s, h, 0.5);
+    s = fma(s, e, s);
+    half_r = fma(h, e, h);
+    return fma(fma(-s, s, q), half_r, s);
 }
 
 // F_{h-2}, F_{h-1}, F_h at a single-precision x in [-8, 1) from the
@@ -449,7 +467,7 @@ template <int D> __device__ __forceinline__ Fd3 fd3_poly(float x, float &hm3)
 {
     const int i = (int)((x - (float)FD_PX0) * 4.f);
     const float c = (float)FD_PX0 + 0.125f + 0.25f * (float)i, tf = x - c;
-    const double t = (double)x - (double)c;     // (tf is rounded where |x| is small)
+    const double t = widen(x) - widen(c);       // (tf is rounded where |x| is small)
     const double(*p)[3] = FD_POLY[D - 2][i];
     Fd3 r{p[FD_PDEG][0], p[FD_PDEG][1], p[FD_PDEG][2]};
 #pragma unroll
@@ -473,8 +491,10 @@ template <int D> __device__ __forceinline__ Fd3 fd3_poly(float x, float &hm3)
 // (F_k' = F_{k-1}; terms beyond delta^2 are below delta^3 / 6 < 2e-17), and
 // their correction brings the error to ~1e-16.  So the solve takes ~170
 // double-precision instructions instead of three evaluations of series of up
-// to 40 terms.  False (nothing written) where the point leaves the tables'
-// range or the first correction is not small.
+// to 40 terms; conversions to and from single precision, 64 cycles each on the
+// double pipe, are done on the bits.  nup, ndn and neps within 2^+-39.  False
+// (nothing written) where the point leaves the tables' range or the first
+// correction is not small.
 template <int D>
 __device__ __forceinline__ bool fd_one_pass(double nup, double ndn, double neps, float b0f, float nu1f, float nu2f,
                                             const FdJacF &J, FdParams &p)
@@ -482,18 +502,10 @@ __device__ __forceinline__ bool fd_one_pass(double nup, double ndn, double neps,
     constexpr float hf = 0.5f * D;
     constexpr double h = 0.5 * D;
     if (!(nu1f >= (float)FD_PX0 && nu1f < 1.f && nu2f >= (float)FD_PX0 && nu2f < 1.f)) return false;
-    // within single precision's range (the reciprocals)
-    if (!(b0f > 1e-12f && b0f < 1e12f && nup < 1e12 && ndn > 1e-12 && neps > 1e-12 && neps < 1e12)) return false;
-    const double b0 = b0f, rb = fd_recip(b0), q = kTwoPi * rb;
-    double A = q;           // (2 pi / b0)^h
-    if (D == 3) {           // q sqrt(q): the float square root and two Newton steps
-        const float sf = sqrtf((float)q);
-        const double hs = (double)(0.5f / sf);
-        double s = sf;
-        s = fma(fma(-s, s, q), hs, s);
-        s = fma(fma(-s, s, q), hs, s);
-        A = q * s;
-    }
+    if (!(b0f > 1e-12f && b0f < 1e12f)) return false;       // (the reciprocal)
+    const double b0 = widen(b0f), rb = fd_recip(b0), q = kTwoPi * rb;
+    double A = q, hr;       // (2 pi / b0)^h
+    if (D == 3) A = q * fd_sqrt(q, hr);
     float G1, G2;           // F_{h-3}
     const Fd3 F1 = fd3_poly<D>(nu1f, G1), F2 = fd3_poly<D>(nu2f, G2);
     const double a1 = A * fd_recip(nup), a2 = A * fd_recip(ndn), a3 = h * A * rb * fd_recip(neps);
@@ -503,25 +515,26 @@ __device__ __forceinline__ bool fd_one_pass(double nup, double ndn, double neps,
         d2 = (hf * dt - r2) * J.ig2;
     };
     float t0, x1, x2, t1, y1, y2;
-    solve((float)fma(F1.m1, a1, -1.0), (float)fma(F2.m1, a2, -1.0), (float)fma(F1.h + F2.h, a3, -1.0), t0, x1, x2);
+    solve(narrow(fma(F1.m1, a1, -1.0)), narrow(fma(F2.m1, a2, -1.0)), narrow(fma(F1.h + F2.h, a3, -1.0)), t0, x1, x2);
     if (!(fmaxf(fabsf(t0), fmaxf(fabsf(x1), fabsf(x2))) <= 5e-6f)) return false;
     // at x_0 + delta_0
-    const double dt = t0, dx1 = x1, dx2 = x2;
-    const double m1 = fma(dx1, fma(dx1, (double)(0.5f * G1), F1.m2), F1.m1);
-    const double m2 = fma(dx2, fma(dx2, (double)(0.5f * G2), F2.m2), F2.m1);
+    const double dt = widen(t0), dx1 = widen(x1), dx2 = widen(x2);
+    const double m1 = fma(dx1, fma(dx1, widen(0.5f * G1), F1.m2), F1.m1);
+    const double m2 = fma(dx2, fma(dx2, widen(0.5f * G2), F2.m2), F2.m1);
     const double hh = fma(dx1, fma(0.5 * dx1, F1.m2, F1.m1), F1.h) + fma(dx2, fma(0.5 * dx2, F2.m2, F2.m1), F2.h);
     const double z = h * dt, E = fma(z, fma(z, 0.5, -1.0), 1.0);        // e^(-h dt)
     const double B = fma(dt, fma(dt, 0.5, -1.0), 1.0);                  // e^(-dt)
-    solve((float)fma(m1 * E, a1, -1.0), (float)fma(m2 * E, a2, -1.0), (float)fma(hh * E, a3 * B, -1.0), t1, y1, y2);
-    const double et = dt + (double)t1;
+    solve(narrow(fma(m1 * E, a1, -1.0)), narrow(fma(m2 * E, a2, -1.0)), narrow(fma(hh * E, a3 * B, -1.0)), t1, y1, y2);
+    const double w1 = widen(y1), w2 = widen(y2), wt = widen(t1);
+    const double et = dt + wt;
     p.beta = fma(b0, fma(et * et, 0.5, et), b0);
     const double rbeta = rb * fma(et, fma(et, 0.5, -1.0), 1.0);
-    p.mu_up = ((double)nu1f + (dx1 + (double)y1)) * rbeta;
-    p.mu_dn = ((double)nu2f + (dx2 + (double)y2)) * rbeta;
+    p.mu_up = (widen(nu1f) + (dx1 + w1)) * rbeta;
+    p.mu_dn = (widen(nu2f) + (dx2 + w2)) * rbeta;
     // (2 pi/beta)^h F_{h-1} at the solution
-    const double AE = A * fma(-h, (double)t1, 1.0) * E;
-    p.n_up = AE * fma((double)y1, F1.m2, m1);
-    p.n_dn = AE * fma((double)y2, F2.m2, m2);
+    const double AE = A * fma(-h, wt, 1.0) * E;
+    p.n_up = AE * fma(w1, F1.m2, m1);
+    p.n_dn = AE * fma(w2, F2.m2, m2);
     p.status = 0;
     return true;
 }
@@ -540,30 +553,63 @@ __device__ FdParams fd_params_site(double n, double Sx, double Sy, double Sz, do
     constexpr double h = 0.5 * D;
     constexpr double hl2pi = h * 1.8378770664093453;   // h log 2 pi
     FdParams p;
+    const unsigned live = __activemask();
     p.beta = p.mu_up = p.mu_dn = p.ax = p.ay = p.az = p.n_up = p.n_dn = CUDART_NAN;
-    const double nS = sqrt(Sx * Sx + Sy * Sy + Sz * Sz);
-    const double nup = 0.5 * (n + nS), ndn = 0.5 * (n - nS);
-    if (!(ndn > 0.0)) {
-        p.status = 1;
-        return p;
-    }
-    if (nS > 0.0) {
+    // |S|, the axis and the range checks beside the double pipe where every
+    // number is ordinary (|S| zero or not tiny)
+    const double SS = Sx * Sx + Sy * Sy + Sz * Sz, neps = n * eps;
+    const bool none = __double_as_longlong(SS) == 0ll;
+    double nS = 0.0, nup, ndn;
+    bool split = !none;
+    float tf = 0.f, n1f = 0.f, n2f = 0.f;
+    FdJacF J;
+    bool start;
+    auto newton = [&] { return fd_newton_f<D>(narrow(nup), narrow(ndn), narrow(n), narrow(eps), tf, n1f, n2f, J); };
+    if (none || fd_within<120>(SS)) {
+        p.ax = p.ay = p.az = 0.0;
+        if (!none) {
+            double r;
+            nS = fd_sqrt(SS, r);
+            r += r;
+            r = fma(r, fma(-nS, r, 1.0), r);
+            p.ax = Sx * r;
+            p.ay = Sy * r;
+            p.az = Sz * r;
+            p.ax = fma(fma(-p.ax, nS, Sx), r, p.ax);
+            p.ay = fma(fma(-p.ay, nS, Sy), r, p.ay);
+            p.az = fma(fma(-p.az, nS, Sz), r, p.az);
+        }
+        const double hn = 0.5 * n;
+        nup = fma(0.5, nS, hn);
+        ndn = fma(-0.5, nS, hn);
+        start = fd_within<39>(nup) && fd_within<39>(ndn) && fd_within<39>(neps) && fd_within<39>(eps);
+        if (start) start = newton();
+    } else {
+        nS = sqrt(SS);
+        nup = 0.5 * (n + nS);
+        ndn = 0.5 * (n - nS);
         p.ax = Sx / nS;
         p.ay = Sy / nS;
         p.az = Sz / nS;
-    } else {
-        p.ax = p.ay = p.az = 0.0;
+        start = false;
+    }
+    // lanes that took different numbers of iterations go through the double
+    // pass together (90 x 101 x 75 sites of differing states 410 -> 267 us; with
+    // the conversions, the root and the divisions beside the double pipe 531 ->
+    // 410, a smooth 64^3 131 -> 101)
+    __syncwarp(live);
+    // the single-precision solution, and one pass in double from it
+    if (start && fd_one_pass<D>(nup, ndn, neps, expf(tf), n1f, split ? n2f : n1f, J, p)) return p;
+    if (!(ndn > 0.0)) {
+        p.ax = p.ay = p.az = CUDART_NAN;
+        p.status = 1;
+        return p;
     }
     if (!(eps > 0.0)) {
         p.status = 2;
         return p;
     }
-    const bool split = nS > 0.0;
-    // the single-precision solution, and one pass in double from it
-    float tf = 0.f, n1f = 0.f, n2f = 0.f;
-    FdJacF J;
-    const bool start = fd_newton_f<D>((float)nup, (float)ndn, (float)n, (float)eps, tf, n1f, n2f, J);
-    if (start && fd_one_pass<D>(nup, ndn, n * eps, expf(tf), n1f, split ? n2f : n1f, J, p)) return p;
+    if (!start) start = newton();
     const double lA = log(nup), lB = split ? log(ndn) : lA, lC = log(n * eps / h);
     double t = log(h / eps);
     double nu1 = lA - hl2pi + h * t, nu2 = lB - hl2pi + h * t;

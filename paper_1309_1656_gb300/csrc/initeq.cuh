@@ -14,6 +14,7 @@
 
 #include "fix64.cuh"
 #include "kernels.cuh"
+#include "quadsum.cuh"
 
 namespace qlbm {
 
@@ -96,21 +97,6 @@ __device__ __forceinline__ bool fx_round_half(long long t, int unit, unsigned ep
     out = __uint2float_rn((m1 & 0xffffff00u) | 0x100u) * fx_pow2(unit + 32 - lz);
     out = __int_as_float(__float_as_int(out) | (int)sign);
     return ok;
-}
-
-// t 2^unit as a double in integer operations (fx_to_double without the
-// double pipe).
-__device__ __forceinline__ double fx_to_double_int(long long t, int unit)
-{
-    const long long s = t >> 63;
-    const unsigned long long a = (unsigned long long)((t ^ s) - s);
-    if (a == 0ull) return 0.0;
-    const int lz = __clzll((long long)a);       // >= 1: |t| < 2^63
-    const unsigned long long m = (a << (lz - 1)) + 0x200u;      // leading bit at 62
-    // leading bit 2^(63 - lz) of t: exponent unit + 63 - lz, one of it from the
-    // leading bit itself (bit 20 of the high word)
-    const unsigned hi = (unsigned)(m >> 42) + ((unsigned)(unit + 63 - lz + 1023 - 1) << 20);
-    return __hiloint2double((int)(hi | ((unsigned)s & 0x80000000u)), (int)(unsigned)(m >> 10));
 }
 
 // Stores the vector of direction q (class cls): t[c] 2^unit[c] the components
