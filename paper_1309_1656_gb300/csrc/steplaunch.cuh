@@ -56,10 +56,17 @@ cudaError_t Launchers<D, Codec>::step_fd(qlbm_ctx *h, bool odd)
         // matrices, the fixed-point step reads them: 96 bytes per site and a
         // second read of the state, against a solve held up by the one-kernel
         // form's ~600 other double-precision instructions.  D3Q19 64^3: 677 ->
-        // 207 us.  Without room for the matrices, or at omega > 2: one kernel.
-        if (!h->fd_rho && cudaMalloc(&h->fd_rho, (size_t)h->g.N * sizeof(DQuad)) != cudaSuccess) {
-            cudaGetLastError();
-            h->fd_rho = nullptr;
+        // 180 us.  Without room for the matrices, or at omega > 2: one kernel.
+        // (The caller may be capturing this thread's work: the allocation is
+        // not part of it.)
+        if (!h->fd_rho) {
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            if (cudaMalloc(&h->fd_rho, (size_t)h->g.N * sizeof(DQuad)) != cudaSuccess) {
+                cudaGetLastError();
+                h->fd_rho = nullptr;
+            }
+            cudaThreadExchangeStreamCaptureMode(&mode);
         }
         FixConst fc;
         if (h->fd_rho && make_fix_const(h->hc, h->dt / h->tau, &fc)) {
