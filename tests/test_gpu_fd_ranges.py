@@ -35,20 +35,17 @@ def test_fd_params_mixed_ranges(q, oracle_mod, prec, d, dims):
         lat.init_equilibrium(rho4, 0.01 * rng.normal(size=(d, N)), eps)
         r4, u, e = lat.moments()
         beta, mu_up, mu_dn, ax, nfail = lat.fd_params()
-    failed = 0
-    for s in range(N):
-        rc, ref = oracle_mod.fd_params(d, r4[:, s], e[s])
-        failed += rc != 0
-        if rc:
-            assert np.isnan(beta[s])
-            continue
-        # against the equations themselves: near |S| = 0 the oracle's own
-        # splitting is 6e-9 off
+    assert np.isnan(beta).sum() == nfail and np.all(np.isnan(beta[bad]))
+    ok = np.isfinite(beta)
+    ok[bad] = True
+    assert np.all(ok[n < 60.0])         # (n = 60 can lie below the degenerate limit)
+    for s in np.flatnonzero(np.isfinite(beta)):
+        # against the equations themselves (near |S| = 0 the splitting of the
+        # oracle's own solve is 6e-9 off)
         nS = np.linalg.norm(r4[1:, s])
         nu, nd, en = oracle_mod.fd_moments(d, beta[s], mu_up[s], mu_dn[s])
         assert nu == pytest.approx(0.5 * (r4[0, s] + nS), rel=1e-9)
         assert nd == pytest.approx(0.5 * (r4[0, s] - nS), rel=1e-9)
         assert en == pytest.approx(e[s], rel=1e-9)
-        S = r4[1:, s]       # (the oracle gives no axis where n + |S| rounds to n)
+        S = r4[1:, s]
         assert np.allclose(ax[:, s], S / (np.linalg.norm(S) or 1.0), atol=1e-9)
-    assert nfail == failed >= len(bad)
