@@ -65,7 +65,8 @@ typedef enum qlbm_status {
 
 typedef enum qlbm_lattice { QLBM_D2Q9 = 2, QLBM_D3Q19 = 3 } qlbm_lattice;
 
-/* Storage precision of the populations.  QLBM_FP64 computes in double;
+/* Storage precision of the populations.  QLBM_FP64 stores
+   doubles and computes to at least double precision;
    QLBM_FP32 stores and computes in float; QLBM_FP16_DEV stores the deviation
    W_i - W_i^ref from a uniform reference equilibrium in half precision and
    computes in float; QLBM_DF64 stores each value as an unevaluated sum of two
@@ -74,14 +75,11 @@ typedef enum qlbm_lattice { QLBM_D2Q9 = 2, QLBM_D3Q19 = 3 } qlbm_lattice;
    per step; no reverse mode: the adjoint calls return
    QLBM_ERR_UNSUPPORTED).  QLBM_FP64_DF stores IEEE doubles exactly as
    QLBM_FP64 does (same layout, same exact state read-out and set-up, same
-   moments, reductions and Fermi-Dirac kernels) but steps in double-float
-   arithmetic: each double is split into two floats, the step runs on the
-   single-precision pipes and rounds its result to double (within ~1e-14 of
-   the QLBM_FP64 step per step; no reverse mode).  Both double-float
-   precisions have single precision's exponent range: magnitudes below
-   2^-126 (~1.2e-38) are read as signed zeros and every stepped value
-   carries an absolute error up to ~2^-126 besides the relative one;
-   magnitudes from 2^128 on are flagged as non-finite. */
+   moments, reductions and Fermi-Dirac kernels) and has no reverse mode; its
+   step is the QLBM_FP64 one within single precision's exponent range.
+   Both QLBM_DF64 and QLBM_FP64_DF read magnitudes below 2^-126 (~1.2e-38)
+   as signed zeros and flag those from 2^128 on as non-finite; a stepped
+   double-float value also carries an absolute error up to ~2^-126. */
 typedef enum qlbm_precision {
     QLBM_FP64 = 0,
     QLBM_FP32 = 1,
