@@ -417,6 +417,15 @@ inline Chunks make_chunks(const Grid &g)
 }
 constexpr int kFixBlock = 64;
 
+// The chunk of a thread's warp, `threads` per block.  Warps are counted, not
+// threads: 32 threads per chunk wrap 32 bits from 2^27 chunks on (2^30 sites,
+// or 2^27 rows of up to 8), and chunks come up to the 2^31 - 64 sites of a
+// lattice.
+FX_FN int chunk_of_thread(unsigned block, unsigned thread, int threads)
+{
+    return (int)(block * (unsigned)(threads / 32) + (thread >> 5));
+}
+
 __device__ __forceinline__ long long fx_from_lane0(long long v)
 {
     return __shfl_sync(0xffffffffu, v, 0, 4);   // the site's lane 0 (component f)
@@ -560,7 +569,7 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
     constexpr int Q = Lattice<D>::Q;
     const unsigned all = 0xffffffffu;
     wait_for_previous();
-    const int chunk = (int)((blockIdx.x * kFixBlock + threadIdx.x) >> 5);
+    const int chunk = chunk_of_thread(blockIdx.x, threadIdx.x, kFixBlock);
     if (chunk >= ch.total) return;      // the whole warp
     const int c = threadIdx.x & 3;
     const int row = fast_div(chunk, ch.row);

@@ -361,7 +361,7 @@ __global__ void __launch_bounds__(kQuadBlock)
 k_moments(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Codec codec, Chunks ch, QuadRef ref, MomentScale sc,
           double *__restrict__ rho4, double *__restrict__ u, double *__restrict__ eps)
 {
-    const int chunk = (int)((blockIdx.x * kQuadBlock + threadIdx.x) >> 5), c = threadIdx.x & 3;
+    const int chunk = chunk_of_thread(blockIdx.x, threadIdx.x, kQuadBlock), c = threadIdx.x & 3;
     if (chunk >= ch.total) return;      // the whole warp
     SiteIdx si;
     const bool active = quad_site(g, ch, chunk, si);
@@ -417,7 +417,7 @@ k_negative_eq(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Codec c
 {
     constexpr int Q = Lattice<D>::Q;
     const unsigned all = 0xffffffffu;
-    const int chunk = (int)((blockIdx.x * kQuadBlock + threadIdx.x) >> 5), c = threadIdx.x & 3;
+    const int chunk = chunk_of_thread(blockIdx.x, threadIdx.x, kQuadBlock), c = threadIdx.x & 3;
     if (chunk >= ch.total) return;      // the whole warp
     SiteIdx si;
     const bool active = quad_site(g, ch, chunk, si);
@@ -475,12 +475,14 @@ k_conserved_partial(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, C
                     double *__restrict__ partials)
 {
     const unsigned all = 0xffffffffu;
-    const int c = threadIdx.x & 3, nw = (int)gridDim.x * (kRedBlock / 32);
+    const int c = threadIdx.x & 3;
+    const unsigned nw = gridDim.x * (kRedBlock / 32);
     double acc[2] = {0.0, 0.0};
     wait_for_previous();
-    for (int chunk = (int)((blockIdx.x * kRedBlock + threadIdx.x) >> 5); chunk < ch.total; chunk += nw) {
+    // (unsigned: the step beyond the last chunk can pass 2^31)
+    for (unsigned k = (unsigned)chunk_of_thread(blockIdx.x, threadIdx.x, kRedBlock); k < (unsigned)ch.total; k += nw) {
         SiteIdx si;
-        const bool active = quad_site(g, ch, chunk, si);
+        const bool active = quad_site(g, ch, (int)k, si);
         const QuadSums s = quad_sums<D, Codec, SWAPPED>(pl, g, si, codec, ref);
         double M, v;
         if (s.fine) {

@@ -1,0 +1,21 @@
+// Host entry points to the device headers' arithmetic (functions compiled for
+// both sides), for the checks that need no GPU: loaded by
+// test_host_arithmetic.py.
+#include "../paper_1309_1656_gb300/csrc/fix64.cuh"
+
+using namespace qlbm;
+
+// The chunks that the warps of block `block` take, and the number of blocks a
+// launch over `nx` x `rows` sites has.
+extern "C" int chunk_of_warp(unsigned block, unsigned warp, int threads)
+{
+    return chunk_of_thread(block, 32 * warp + 31, threads);
+}
+extern "C" int chunks_of_lattice(int nx, int rows)
+{
+    Grid g = {};
+    g.nx = nx;
+    g.ny = rows;
+    g.nz = 1;
+    return make_chunks(g).total;
+}
