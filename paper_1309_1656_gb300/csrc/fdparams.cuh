@@ -461,11 +461,19 @@ __device__ __forceinline__ double fd_sqrt(double q, double &half_r)
     return fma(fma(-s, s, q), half_r, s);
 }
 
+// The interval of the polynomial tables for x in [-8, 1).  x + 8 is rounded:
+// for the last 2^-21 below 1 it gives 9, the end of the last interval.
+__host__ __device__ __forceinline__ int fd_interval(float x)
+{
+    const int i = (int)((x - (float)FD_PX0) * 4.f);
+    return i < FD_PINT ? i : FD_PINT - 1;
+}
+
 // F_{h-2}, F_{h-1}, F_h at a single-precision x in [-8, 1) from the
 // polynomials on intervals of 1/4; F_{h-3} in single precision.
 template <int D> __device__ __forceinline__ Fd3 fd3_poly(float x, float &hm3)
 {
-    const int i = (int)((x - (float)FD_PX0) * 4.f);
+    const int i = fd_interval(x);
     const float c = (float)FD_PX0 + 0.125f + 0.25f * (float)i, tf = x - c;
     const double t = widen(x) - widen(c);       // (tf is rounded where |x| is small)
     const double(*p)[3] = FD_POLY[D - 2][i];

@@ -1,6 +1,7 @@
 // Host entry points to the device headers' arithmetic (functions compiled for
 // both sides), for the checks that need no GPU: loaded by
 // test_host_arithmetic.py.
+#include "../paper_1309_1656_gb300/csrc/fdparams.cuh"
 #include "../paper_1309_1656_gb300/csrc/fix64.cuh"
 
 using namespace qlbm;
@@ -19,3 +20,9 @@ extern "C" int chunks_of_lattice(int nx, int rows)
     g.nz = 1;
     return make_chunks(g).total;
 }
+
+// Interval of the Fermi-Dirac polynomial tables, their number, and the
+// distance of x from the interval's centre (1/8 at most).
+extern "C" int fd_table_interval(float x) { return fd_interval(x); }
+extern "C" int fd_table_intervals() { return FD_PINT; }
+extern "C" double fd_table_offset(float x) { return (double)x - (FD_PX0 + 0.125 + 0.25 * fd_interval(x)); }

@@ -49,3 +49,26 @@ def test_fd_params_mixed_ranges(q, oracle_mod, prec, d, dims):
         assert en == pytest.approx(e[s], rel=1e-9)
         S = r4[1:, s]
         assert np.allclose(ax[:, s], S / (np.linalg.norm(S) or 1.0), atol=1e-9)
+
+
+@pytest.mark.parametrize("d,dims", [(2, (41, 3, 1)), (3, (33, 2, 3))])
+def test_fd_params_at_the_ends_of_the_tables(q, oracle_mod, d, dims):
+    # beta mu spread over 2^-20 on both sides of 1 and of -8, where the
+    # polynomials begin and end; the bound of the ordinary comparison, 1e-9
+    N = int(np.prod(dims))
+    rng = np.random.default_rng(40 + d)
+    nu = rng.choice([1.0, -8.0], (2, N)) + rng.integers(-16, 17, (2, N)) * 2.0**-24
+    beta = rng.uniform(0.9, 1.1, N)
+    axis = np.zeros((3, N))
+    axis[2] = 1.0
+    with q.Lattice(d, dims, 0.8, 1.0, precision="fp64") as lat:
+        q.qlbm_init_fd_params(lat.h, beta, nu[0] / beta, nu[1] / beta, axis, np.zeros((d, N)))
+        r4, u, e = lat.moments()
+        b, mu_up, mu_dn, ax, nfail = lat.fd_params()
+    assert nfail == 0
+    for s in range(N):
+        nS = np.linalg.norm(r4[1:, s])
+        a, c, en = oracle_mod.fd_moments(d, b[s], mu_up[s], mu_dn[s])
+        assert a == pytest.approx(0.5 * (r4[0, s] + nS), rel=1e-9)
+        assert c == pytest.approx(0.5 * (r4[0, s] - nS), rel=1e-9)
+        assert en == pytest.approx(e[s], rel=1e-9)

@@ -4,6 +4,7 @@ import ctypes
 import os
 import subprocess
 
+import numpy as np
 import pytest
 
 from paper_1309_1656_gb300 import _build
@@ -33,3 +34,17 @@ def test_every_chunk_has_one_warp(host, nx, rows, threads):
         for warp in range(per_block):
             # (a warp beyond the last chunk must see a number not below total)
             assert host.chunk_of_warp(ctypes.c_uint(block), ctypes.c_uint(warp), threads) == block * per_block + warp
+
+
+def test_fermi_dirac_intervals_end_inside_the_tables(host):
+    # every float of the last 2^-18 below 1, those around -8 and the seams
+    host.fd_table_offset.restype = ctypes.c_double
+    ends = [np.float32(1.0)] + [np.float32(-8.0 + 0.25 * i) for i in range(36)]
+    xs = [v for e in ends for v in (e, np.nextafter(e, np.float32(9)), np.nextafter(e, np.float32(-9)))]
+    xs += list(1.0 - np.arange(1, 65) * np.float32(2.0**-24))
+    n = host.fd_table_intervals()
+    for x in map(float, xs):
+        if -8.0 <= x < 1.0:
+            assert 0 <= host.fd_table_interval(ctypes.c_float(x)) < n
+            # (a point at a seam may fall to either side of it by rounding)
+            assert abs(host.fd_table_offset(ctypes.c_float(x))) <= 0.125 + 2.0**-20
