@@ -351,6 +351,14 @@ inline Dd reciprocal(Dd a)
     return r + r * (Dd(1.0) + -(a * r));
 }
 
+// Host: 1 - omega in q62 for omega in [0, 2] (omega - 1 is exact from 1 on,
+// and neither branch leaves 64 bits: 2.0 itself is 2^63).
+inline long long fx_one_minus(double omega)
+{
+    const double q62 = 4611686018427387904.0;
+    return omega < 1.0 ? kFxOne - llrint(omega * q62) : -llrint((omega - 1.0) * q62);
+}
+
 // Host: the constants, false where they leave the form's range (then the
 // double-precision kernel steps the lattice).
 inline bool make_fix_const(const HostConsts &k, double omega, FixConst *o)
@@ -364,8 +372,7 @@ inline bool make_fix_const(const HostConsts &k, double omega, FixConst *o)
     };
     const double q62 = 4611686018427387904.0;
     const Dd K(k.K), c(k.c), inv = reciprocal(Dd(k.m) + -(c * c)), om(omega);
-    const long long omc = kFxOne - (omega < 1.0 ? llrint(omega * q62) : 2 * llrint(omega * q62 * 0.5));
-    o->omc = fx_split(omc);
+    o->omc = fx_split(fx_one_minus(omega));
     for (int m = 0; m < 3; ++m) {
         const Dd ow = om * Dd(k.w[m]);
         o->al[m] = fix(ow, q62, 1.0);

@@ -26,3 +26,6 @@ extern "C" int chunks_of_lattice(int nx, int rows)
 extern "C" int fd_table_interval(float x) { return fd_interval(x); }
 extern "C" int fd_table_intervals() { return FD_PINT; }
 extern "C" double fd_table_offset(float x) { return (double)x - (FD_PX0 + 0.125 + 0.25 * fd_interval(x)); }
+
+// 1 - omega as the FP64 step's constants hold it (q62).
+extern "C" long long one_minus_omega(double omega) { return fx_one_minus(omega); }

@@ -1,8 +1,10 @@
 """Index and number arithmetic of the kernels, run on the host: sizes that no
 test could allocate, and comparisons with exact arithmetic."""
 import ctypes
+import fractions
 import os
 import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -10,13 +12,17 @@ import pytest
 from paper_1309_1656_gb300 import _build
 
 
+def compile_host(path, flags="-fPIC"):
+    here = os.path.dirname(os.path.abspath(__file__))
+    lib = str(path / "libhost.so")
+    subprocess.run([_build.nvcc(), "-O2", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", flags, "-shared",
+                    "-I", _build.INCLUDE, os.path.join(here, "host_kernels.cu"), "-o", lib], check=True)
+    return lib
+
+
 @pytest.fixture(scope="module")
 def host(tmp_path_factory):
-    here = os.path.dirname(os.path.abspath(__file__))
-    lib = str(tmp_path_factory.mktemp("host") / "libhost.so")
-    subprocess.run([_build.nvcc(), "-O2", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC", "-shared",
-                    "-I", _build.INCLUDE, os.path.join(here, "host_kernels.cu"), "-o", lib], check=True)
-    return ctypes.CDLL(lib)
+    return ctypes.CDLL(compile_host(tmp_path_factory.mktemp("host")))
 
 
 # rows of at most one chunk, rows of two, and square lattices, around the
@@ -48,3 +54,20 @@ def test_fermi_dirac_intervals_end_inside_the_tables(host):
             assert 0 <= host.fd_table_interval(ctypes.c_float(x)) < n
             # (a point at a seam may fall to either side of it by rounding)
             assert abs(host.fd_table_offset(ctypes.c_float(x))) <= 0.125 + 2.0**-20
+
+
+OMEGAS = [0.0, 2.0**-60, 0.1, 0.5, 1.0 - 2.0**-53, 1.0, 1.0 + 2.0**-52, 1.25, 1.9, 2.0 - 2.0**-52, 2.0]
+
+
+def test_one_minus_omega(host):
+    host.one_minus_omega.restype = ctypes.c_longlong
+    for omega in OMEGAS:
+        want = (1 - fractions.Fraction(omega)) * 2**62
+        assert abs(host.one_minus_omega(ctypes.c_double(omega)) - want) <= 1
+
+
+def test_one_minus_omega_stays_within_64_bits(tmp_path):
+    # signed overflow traps in this build (in a process of its own)
+    lib = compile_host(tmp_path, "-fPIC,-fsanitize=signed-integer-overflow,-fsanitize-undefined-trap-on-error")
+    code = "import ctypes; f = ctypes.CDLL(%r).one_minus_omega; [f(ctypes.c_double(w)) for w in %r]" % (lib, OMEGAS)
+    assert subprocess.run([sys.executable, "-c", code]).returncode == 0
