@@ -838,10 +838,6 @@ int qlbm_set_magnetic_field(qlbm_handle h, double mu, const double B[3])
                              y * x * C + z * s, c + y * y * C,     y * z * C - x * s,
                              z * x * C - y * s, z * y * C + x * s, c + z * z * C};
         for (int i = 0; i < 9; ++i) rot[i] = r[i];
-        h->quat[0] = cos(0.5 * th);
-        h->quat[1] = sin(0.5 * th) * x;
-        h->quat[2] = sin(0.5 * th) * y;
-        h->quat[3] = sin(0.5 * th) * z;
         mag = 1;
     }
     for (int i = 0; i < 9; ++i) h->rot[i] = rot[i];

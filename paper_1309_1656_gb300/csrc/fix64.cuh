@@ -23,7 +23,10 @@
 //
 // Each result errs by at most ~1.2 x 2^-53 of its component's largest value
 // at the site (0.13 rms; the double-precision step, which rounds h, h M - W
-// and W', by up to 8 x 2^-53, 0.5 rms, at omega = 0.5, and more above).
+// and W', by up to 8 x 2^-53, 0.5 rms, at omega = 0.5, and more above).  At
+// smaller omega the double step is more accurate than that on populations
+// small beside the largest; there the last line is done in double
+// (fix_double_below).
 // Warps with a site outside the form's range (non-finite or extreme values,
 // n <= 0, |j| >= 3/8, E2/n a unit off, |h| >= 1) step in double, with the same
 // flags as k_step_aa.
@@ -154,6 +157,7 @@ struct FixConst {
     FxSplit ga[2];          // q62, rest and axis class
     FxSplit c3, c4;         // q62
     long long d0;           // q60
+    int h_unit;             // h_i as formed: units of 2^h_unit
     int valid;              // 0: every site in double
 };
 constexpr long long kFxOne = 1LL << 62;   // 1.0 in q62
@@ -196,6 +200,21 @@ FX_FN double fx_to_double(long long t, int shift)
 #else
     return ldexp(v, shift / (1 << 20));
 #endif
+}
+
+// t 2^unit as a double in integer operations (fx_to_double without the
+// double pipe).
+__device__ __forceinline__ double fx_to_double_int(long long t, int unit)
+{
+    const long long s = t >> 63;
+    const unsigned long long a = (unsigned long long)((t ^ s) - s);
+    if (a == 0ull) return 0.0;
+    const int lz = __clzll((long long)a);       // >= 1: |t| < 2^63
+    const unsigned long long m = (a << (lz - 1)) + 0x200u;      // leading bit at 62
+    // leading bit 2^(63 - lz) of t: exponent unit + 63 - lz, one of it from the
+    // leading bit itself (bit 20 of the high word)
+    const unsigned hi = (unsigned)(m >> 42) + ((unsigned)(unit + 63 - lz + 1023 - 1) << 20);
+    return __hiloint2double((int)(hi | ((unsigned)s & 0x80000000u)), (int)(unsigned)(m >> 10));
 }
 
 // omc X + h m in units of 4 U, rounded to nearest but for the products of the
@@ -360,11 +379,19 @@ inline long long fx_one_minus(double omega)
 }
 
 // Host: the constants, false where they leave the form's range (then the
-// double-precision kernel steps the lattice).
-inline bool make_fix_const(const HostConsts &k, double omega, FixConst *o)
+// double-precision kernel steps the lattice).  normalise: h_i for omega 2^k in
+// [1/2, 1) instead of a smaller omega, so that it keeps its digits (for the
+// update in double, which takes it in units of 2^-(62 + k)).
+inline bool make_fix_const(const HostConsts &k, double omega, bool normalise, FixConst *o)
 {
     *o = FixConst{};
     if (!(omega > 0.0 && omega <= 2.0)) return false;
+    o->h_unit = -62;
+    if (normalise && omega < 0.5) {
+        int e;
+        omega = frexp(omega, &e);
+        o->h_unit += e;
+    }
     bool ok = k.w[2] * (k.d == 3 ? 2.0 : 4.0) == k.w[1];     // the diagonal class is shifts of the axis class
     auto fix = [&](Dd v, double scale, double lim) {
         ok = ok && v.h < lim && v.h > -lim;
@@ -439,54 +466,73 @@ __device__ __forceinline__ long long fx_from_lane0(long long v)
 }
 
 // The magnetic-field term: the rotation of the spins by the unit quaternion
-// (w, x, y, z) (FIELD_UNIFORM: uq, FIELD_SITE: of site s).  Lane c = 1..3 holds
-// component c; in cyclic order p, q, r = its own component of the vector part,
-// the next and the one after, its row of the rotation matrix is
-//   1 - 2 (q^2 + r^2)  (own),  2 (p q - w r)  (next),  2 (p r + w q)  (after).
-// For the uniform field the host gives each lane's row (in the same order) in
-// q62 and (1 - omega) times it; row 0 is the identity's.
+// (w, x, y, z) of site s.  Lane c = 1..3 holds component c; in cyclic order
+// p, q, r = its own component of the vector part, the next and the one after,
+// its row of the rotation matrix is
+//   1 - 2 (q^2 + r^2)  (own),  2 (p q - w r)  (next),  2 (p r + w q)  (after);
+// lane 0 (f) has the identity's.  For the uniform field the host gives each
+// lane's row in that order.
 struct FixField {
-    double v[4];        // (w, x, y, z)
-    FxSplit r[4][3], m[4][3];
+    double r[4][3];
 };
-inline void make_fix_field(const double (&rot)[9], const double (&quat)[4], double omega, FixField *o)
+inline void make_fix_field(const double (&rot)[9], FixField *o)
 {
-    auto q62 = [](Dd v) { return fx_split(llrint(v.h * 4611686018427387904.0) + llrint(v.l * 4611686018427387904.0)); };
-    const Dd omc = Dd(1.0) + Dd(-omega);
-    for (int i = 0; i < 4; ++i) o->v[i] = quat[i];
     for (int c = 0; c < 4; ++c)
-        for (int b = 0; b < 3; ++b) {
-            const double r = c ? rot[3 * (c - 1) + (c - 1 + b) % 3] : (b ? 0.0 : 1.0);
-            o->r[c][b] = q62(Dd(r));
-            o->m[c][b] = q62(omc * Dd(r));
-        }
+        for (int b = 0; b < 3; ++b) o->r[c][b] = c ? rot[3 * (c - 1) + (c - 1 + b) % 3] : (b ? 0.0 : 1.0);
 }
 FX_FN int fx_next_lane(int c) { return c == 3 ? 1 : c + 1; }
 FX_FN int fx_prev_lane(int c) { return c <= 1 ? 3 : c - 1; }
 template <int FIELD>
-__device__ __forceinline__ void fx_load_quat(const FixField &uq, const DQuad *qf, int s, int c, double (&o)[4])
+__device__ __forceinline__ void fx_rotation_row(const FixField &uq, const DQuad *qf, int s, int c, double (&r)[3])
 {
-    const int p = c ? c : 1;
-    const double *v = FIELD == FIELD_SITE ? reinterpret_cast<const double *>(qf + s) : uq.v;
-    o[0] = v[0];
-    o[1] = v[p];
-    o[2] = v[fx_next_lane(p)];
-    o[3] = v[fx_prev_lane(p)];
+    if constexpr (FIELD == FIELD_SITE) {
+        const double *v = reinterpret_cast<const double *>(qf + s);
+        const int own = c ? c : 1;
+        const double w = v[0], p = v[own], q = v[fx_next_lane(own)], t = v[fx_prev_lane(own)];
+        r[0] = 1.0 - 2.0 * (q * q + t * t);
+        r[1] = 2.0 * (p * q - w * t);
+        r[2] = 2.0 * (p * t + w * q);
+        if (c == 0) {
+            r[0] = 1.0;
+            r[1] = r[2] = 0.0;
+        }
+    } else if constexpr (FIELD == FIELD_UNIFORM) {
+#pragma unroll
+        for (int b = 0; b < 3; ++b) r[b] = uq.r[c][b];
+    } else {
+        r[0] = r[1] = r[2] = 0.0;
+    }
 }
-// A number of magnitude <= 1 in q62.
-__device__ __forceinline__ FxSplit fx_unit(double v)
+// The exponent of a rotated component.  The three components (own, next,
+// after) keep alignments e[b] of their own; the result is in units of
+// 2^(E - 1080) with 2^E at least sum_b |r_b| 2^e_b and at most twice that, so
+// that a component small beside the others keeps its digits as far as the
+// rotation does not mix them in.  e[b] <= 0: the component is zero.
+FX_FN int fx_mixed_exponent(const unsigned (&rh)[3], const int (&e)[3])
 {
-    return fx_split(fx_align((unsigned)__double2hiint(v), (unsigned)__double2loint(v), 1023) << 5);
+    int top = 0, x[3];
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const int er = (int)((rh[b] >> 20) & 0x7ffu);       // |r_b| < 2^(er - 1022)
+        x[b] = er && e[b] > 0 ? e[b] + er - 1022 : -4000;
+        top = x[b] > top ? x[b] : top;
+    }
+    // sum_b |r_b| 2^(e_b - top), each term below 1 (the largest at least 1/2)
+    float t = 0.f;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+        const int k = x[b] - top;
+        if (k > -100) t += fx_float((((rh[b] & 0xfffffu) + 1u) << 3) + (unsigned)((126 + k) << 23));
+    }
+    // (the sum of X_b r_b stays below 2^58 where t 2^top <= 2^E)
+    const int E = top + (t > 1.f ? (t > 2.f ? 2 : 1) : (t > 0.51f ? 0 : -1));
+    return E > 64 ? E : 64;     // (the results' exponents stay positive)
 }
-// The row of the rotation matrix (q62); lane 0: the identity's.
-__device__ __forceinline__ void fx_rotation_row(const double (&fq)[4], int c, FxSplit (&R)[3])
+// r 2^(e - E) in q62 (at most 1).
+FX_FN FxSplit fx_scaled_row(unsigned rh, unsigned rl, int e, int E)
 {
-    const FxSplit w = fx_unit(fq[0]), p = fx_unit(fq[1]), q = fx_unit(fq[2]), r = fx_unit(fq[3]);
-    const long long d = kFxOne - 8 * (fx_mul(q, q) + fx_mul(r, r));     // q60 products
-    const long long n = 8 * (fx_mul(p, q) - fx_mul(w, r)), a = 8 * (fx_mul(p, r) + fx_mul(w, q));
-    R[0] = fx_split(c ? d : kFxOne);
-    R[1] = fx_split(c ? n : 0);
-    R[2] = fx_split(c ? a : 0);
+    const bool none = ((rh >> 20) & 0x7ffu) == 0u || e <= 0;
+    return fx_split(none ? 0 : fx_align(rh, rl, 1018 + E - e));
 }
 __device__ __forceinline__ FxSplit fx_shfl(FxSplit v, int lane)
 {
@@ -497,10 +543,10 @@ __device__ __forceinline__ FxSplit fx_shfl(FxSplit v, int lane)
 // site outside the fixed-point form; lane c = 0 holds f, 1..3 the spins.
 // FD: the equilibrium is built from the component R of a rebuilt density
 // matrix instead of M (the flag then looks at n only).  FIELD: the spins are
-// rotated by the unit quaternion fq (fx_load_quat).
+// rotated, r the lane's row (fx_rotation_row).
 template <int D, bool FD, bool FIELD>
 __device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[Lattice<D>::Q], const Coll<double> &k,
-                                                      double R, const double (&fq)[4])
+                                                      double R, const double (&r)[3])
 {
     constexpr int Q = Lattice<D>::Q;
     double M = 0.0, J[3] = {0.0, 0.0, 0.0}, E = 0.0;
@@ -531,13 +577,11 @@ __device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[La
     }
     if constexpr (FIELD) {
         const int c = threadIdx.x & 3;
-        const double r0 = 1.0 - 2.0 * (fq[2] * fq[2] + fq[3] * fq[3]), r1 = 2.0 * (fq[1] * fq[2] - fq[0] * fq[3]),
-                     r2 = 2.0 * (fq[1] * fq[3] + fq[0] * fq[2]);
 #pragma unroll
         for (int q = 0; q < Q; ++q) {
             const double v = __longlong_as_double((long long)w[q]);
             const double v1 = __shfl_sync(all, v, fx_next_lane(c), 4), v2 = __shfl_sync(all, v, fx_prev_lane(c), 4);
-            if (c) w[q] = (unsigned long long)__double_as_longlong(r0 * v + r1 * v1 + r2 * v2);
+            if (c) w[q] = (unsigned long long)__double_as_longlong(r[0] * v + r[1] * v1 + r[2] * v2);
         }
     }
     double sum = (threadIdx.x & 3) ? fabs(M) : fabs(be);
@@ -555,10 +599,11 @@ __device__ __forceinline__ unsigned fx_collide_double(unsigned long long (&w)[La
 // the same arithmetic in all three.
 // With FD the equilibrium is built from a density matrix per site (rho, Eq.
 // WeqDiscr) instead of the populations' own; P_i keeps their u and eps.
-// With a field the three spin components share one alignment (|X| < 2^57, so
-// that a rotated sum still fits) and the rotation R is folded into the
-// relaxation: sum_b (1 - omega) R_ab X_b + h (R M)_a, the other two components
-// from the neighbouring lanes.
+// With a field the rotation R is folded into the relaxation: sum_b (1 - omega)
+// R_ab X_b + h (R M)_a, the other two components from the neighbouring lanes,
+// each with its own alignment (fx_mixed_exponent).
+// DBL: the populations are updated in double from the integer sums and
+// coefficients (fix_double_below).
 // rg: the largest high word (magnitude) of a component that counts as zero,
 // and the smallest that is non-finite; QLBM_FP64_DF has single precision's
 // exponent range there (2^-126, 2^128).
@@ -567,7 +612,25 @@ struct FixRange {
 };
 inline FixRange make_fix_range(bool single) { return single ? FixRange{(897u << 20) - 1u, 1151u << 20} : FixRange{0u, ~0u}; }
 enum : int { FIX_EVEN = 0, FIX_ODD = 1, FIX_PUSH = 2 };
-template <int D, int MODE, bool FD, int FIELD>
+// The omega below which the populations are updated in double, two multiply-
+// adds each.  The fixed-point update errs by up to 1.3 x 2^-56 of the
+// component's largest value whatever omega is, the double step by a few 2^-53
+// of omega h M and by 2^-54 of the result: for a population much smaller than
+// the largest the double step is the better one where omega is small.  Root
+// mean square errors of populations between 2^-5 and 2^-4 of the largest, in
+// 2^-53 of themselves, over random sites (D3Q19; fixed point, double step):
+// omega = 1.25: 0.9, 4.4; 0.5: 0.9, 1.8; 0.1: 0.9, 0.5; 0.01: 0.9, 0.4, and in
+// proportion below; where one population outweighs all others the double step
+// gains on it from 0.7 down.  In double D3Q19 128^3 takes 660 us instead of
+// 505, with a field 1436 instead of 702, D2Q9 64^2 2.9 instead of 2.3 (the
+// double pipe; 1485, 2207 and 8.3 with everything in double).  QLBM_FP64_DF
+// with a field, stated to 1e-14 of the largest, keeps the fixed-point update
+// further down.
+inline double fix_double_below(int prec, int field)
+{
+    return prec == QLBM_FP64 || field == FIELD_NONE ? 0.75 : 0.0625;
+}
+template <int D, int MODE, bool FD, int FIELD, bool DBL>
 __global__ void __launch_bounds__(kFixBlock, D == 3 ? 8 : 14)
 k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice<D>::Q> dst, Grid g, FixConst fc,
            Coll<double> k, Chunks ch, FixRange rg, const DQuad *__restrict__ rho, FixField uq,
@@ -604,16 +667,11 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
 #pragma unroll
     for (int q = 0; q < Q; ++q) mx = max(mx, (unsigned)(w[q] >> 32) & 0x7fffffffu);
     unsigned flag = mx >= rg.bad ? FLAG_NONFINITE : 0u;
-    if constexpr (FIELD != FIELD_NONE) {
-        const unsigned m1 = __shfl_sync(all, mx, 1, 4), m2 = __shfl_sync(all, mx, 2, 4), m3 = __shfl_sync(all, mx, 3, 4);
-        if (c) mx = max(m1, max(m2, m3));
-    }
-    // a component that counts as zero is shifted out altogether (eb); with a
-    // field the spins have one bit of headroom
+    // a component that counts as zero is shifted out altogether
     const bool zero = mx <= rg.zero;
-    const int eb = zero ? kFxZeroExp : (int)(mx >> 20) + (FIELD != FIELD_NONE && c ? 1 : 0);
-    double fq[4] = {1.0, 0.0, 0.0, 0.0};
-    if constexpr (FIELD != FIELD_NONE) fx_load_quat<FIELD>(uq, k.qf, si.s, c, fq);
+    const int eb = zero ? kFxZeroExp : (int)(mx >> 20);
+    double r[3];
+    fx_rotation_row<FIELD>(uq, k.qf, si.s, c, r);
     double R = 0.0;
     if (FD) R = reinterpret_cast<const double *>(rho + si.s)[c];
     bool fine = fc.valid && __all_sync(all, zero || (eb >= kFxMinExp && eb <= kFxMaxExp));
@@ -627,46 +685,67 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
         for (int a = 0; a < D; ++a) J[a] = fx_from_lane0(J[a]);
         FixCoef cf;
         fine = __all_sync(all, fx_coefficients<D>(fx_from_lane0(M), J, fx_from_lane0(E), fc, cf));
-        if (fine) {
+        if (fine && DBL) {
+            const double m = FD ? R : fx_to_double(M, zero ? 0 : (eb - 1080) * (1 << 20));
+            if constexpr (FIELD == FIELD_NONE) {
+                fx_each_h<D>(cf, [&](int q, long long h) {
+                    const double v = zero ? 0.0 : __longlong_as_double((long long)w[q]);
+                    w[q] = (unsigned long long)__double_as_longlong(
+                        fma(fx_to_double_int(h, fc.h_unit), m, fma(-k.omega, v, v)));
+                });
+            } else {
+                const int n1 = fx_next_lane(c), n2 = fx_prev_lane(c);
+                // f: (f - omega f) + h n; spins: (1 - omega) R s + h R S
+                const double m1 = __shfl_sync(all, m, n1, 4), m2 = __shfl_sync(all, m, n2, 4), omc = 1.0 - k.omega;
+                const double rm = c ? r[0] * m + r[1] * m1 + r[2] * m2 : m;     // of R S
+#pragma unroll
+                for (int b = 0; b < 3; ++b) r[b] *= omc;
+                if (c == 0) r[0] = -k.omega;
+                fx_each_h<D>(cf, [&](int q, long long h) {
+                    const double v = zero ? 0.0 : __longlong_as_double((long long)w[q]);
+                    const double v1 = __shfl_sync(all, v, n1, 4), v2 = __shfl_sync(all, v, n2, 4);
+                    const double t = fma(r[1], v1, r[2] * v2);
+                    w[q] = (unsigned long long)__double_as_longlong(
+                        fma(fx_to_double_int(h, fc.h_unit), rm, fma(r[0], v, c ? t : v)));
+                });
+            }
+        } else if (fine) {
             if (FD) {       // rho's component in the units of M
                 const int rh = __double2hiint(R), e = (rh >> 20) & 0x7ff;
                 const bool none = e <= eb - 70;     // below U / 2^13
                 fine = __all_sync(all, none || (e < eb + 5 && !zero));
                 M = none ? 0 : __double2ll_rn(__hiloint2double(rh + (1080 - eb) * (1 << 20), __double2loint(R)));
             }
-            const int shift = (eb - 1078) * (1 << 20);
             if constexpr (FIELD == FIELD_NONE) {
+                const int shift = (eb - 1078) * (1 << 20);
                 const FxSplit m = fx_split(M);
                 fx_each_h<D>(cf, [&](int q, long long h) {
                     w[q] = (unsigned long long)__double_as_longlong(
                         fx_to_double(fx_update(X[q], fc.omc, h, m), shift));
                 });
             } else {
-                const int n1 = fx_next_lane(c), n2 = fx_prev_lane(c);
-                FxSplit r[3];
-                if constexpr (FIELD == FIELD_SITE) {
-                    fx_rotation_row(fq, c, r);
-                } else {
+                const int n1 = fx_next_lane(c), n2 = fx_prev_lane(c), e0 = zero ? 0 : eb;
+                const int e[3] = {e0, __shfl_sync(all, e0, n1, 4), __shfl_sync(all, e0, n2, 4)};
+                const unsigned rh[3] = {(unsigned)__double2hiint(r[0]), (unsigned)__double2hiint(r[1]),
+                                        (unsigned)__double2hiint(r[2])};
+                const int E = fx_mixed_exponent(rh, e), shift = (E - 1078) * (1 << 20);
+                FxSplit rt[3];
 #pragma unroll
-                    for (int b = 0; b < 3; ++b) r[b] = uq.r[c][b];
-                }
+                for (int b = 0; b < 3; ++b) rt[b] = fx_scaled_row(rh[b], (unsigned)__double2loint(r[b]), e[b], E);
                 FxSplit m = fx_split(M);
                 const FxSplit m1 = fx_shfl(m, n1), m2 = fx_shfl(m, n2);
-                if (c) m = fx_split((fx_mul(r[0], m) + fx_mul(r[1], m1) + fx_mul(r[2], m2) + 1) << 2);
+                const long long rm = fx_mul(rt[0], m) + fx_mul(rt[1], m1) + fx_mul(rt[2], m2);
+                if (c) m = fx_split(rm ? (rm + 1) << 2 : 0);       // (a zero component stays zero)
 #pragma unroll
-                for (int b = 0; b < 3; ++b) {
-                    if constexpr (FIELD == FIELD_SITE)
-                        r[b] = c ? fx_split(fx_mul(fc.omc, r[b]) << 2) : (b ? FxSplit{0, 0} : fc.omc);
-                    else
-                        r[b] = uq.m[c][b];
-                }
+                for (int b = 0; b < 3; ++b)
+                    rt[b] = c ? fx_split(fx_mul(fc.omc, rt[b]) << 2) : (b ? FxSplit{0, 0} : fc.omc);
                 fx_each_h<D>(cf, [&](int q, long long h) {
                     const FxSplit x = fx_split(X[q]), x1 = fx_shfl(x, n1), x2 = fx_shfl(x, n2), g = fx_split(h);
-                    long long t = fx_mad(x.hi, r[0].lo, fx_mad(x.lo, r[0].hi, 0x80000000LL));
-                    t = fx_mad(x1.hi, r[1].lo, fx_mad(x1.lo, r[1].hi, t));
-                    t = fx_mad(x2.hi, r[2].lo, fx_mad(x2.lo, r[2].hi, t));
+                    long long t = fx_mad(x.hi, rt[0].lo, fx_mad(x.lo, rt[0].hi, 0x80000000LL));
+                    t = fx_mad(x1.hi, rt[1].lo, fx_mad(x1.lo, rt[1].hi, t));
+                    t = fx_mad(x2.hi, rt[2].lo, fx_mad(x2.lo, rt[2].hi, t));
                     t = fx_mad(m.hi, g.lo, fx_mad(m.lo, g.hi, t)) >> 32;
-                    t = fx_mad(x2.hi, r[2].hi, fx_mad(x1.hi, r[1].hi, fx_mad(x.hi, r[0].hi, t)));
+                    t = fx_mad(x2.hi, rt[2].hi, fx_mad(x1.hi, rt[1].hi, fx_mad(x.hi, rt[0].hi, t)));
                     w[q] = (unsigned long long)__double_as_longlong(fx_to_double(fx_mad(m.hi, g.hi, t), shift));
                 });
             }
@@ -675,7 +754,7 @@ k_step_fix(const Planes<double, Lattice<D>::Q> src, const Planes<double, Lattice
     if (!fine) {
 #pragma unroll
         for (int q = 0; q < Q; ++q) w[q] = zero ? 0ull : load(q);
-        flag |= fx_collide_double<D, FD, FIELD != FIELD_NONE>(w, k, R, fq);
+        flag |= fx_collide_double<D, FD, FIELD != FIELD_NONE>(w, k, R, r);
     }
     let_next_start();
     if (active) {

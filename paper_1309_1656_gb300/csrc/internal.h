@@ -75,7 +75,6 @@ struct qlbm_ctx {
     int mag = 0;                        // magnetic-field term: FIELD_NONE, FIELD_UNIFORM or FIELD_SITE
     void *qfield = nullptr;             // per-site field: N unit quaternions (float4, or DQuad for FP64)
     double rot[9] = {1, 0, 0, 0, 1, 0, 0, 0, 1};   // its per-step spin rotation
-    double quat[4] = {1, 0, 0, 0};      // the same as a unit quaternion
     unsigned long long *fd_fail = nullptr;   // device counter of unresolved sites
     void *fd_rho = nullptr;             // density matrices of the step through the parameters (DQuad per site)
     unsigned long long *neg_count = nullptr; // device counter of the negative-equilibrium diagnostic

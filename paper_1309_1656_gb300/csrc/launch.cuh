@@ -83,7 +83,7 @@ inline InitConsts make_init(const qlbm_ctx *h)
 inline FixConst make_fix_unit(const qlbm_ctx *h)
 {
     FixConst fc;
-    make_fix_const(h->hc, 1.0, &fc);
+    make_fix_const(h->hc, 1.0, false, &fc);
     return fc;
 }
 

@@ -173,21 +173,6 @@ __device__ __forceinline__ double quad_double(long long v, int unit)
     return fx_to_double(v, unit * (1 << 20));
 }
 
-// t 2^unit as a double in integer operations (fx_to_double without the
-// double pipe).
-__device__ __forceinline__ double fx_to_double_int(long long t, int unit)
-{
-    const long long s = t >> 63;
-    const unsigned long long a = (unsigned long long)((t ^ s) - s);
-    if (a == 0ull) return 0.0;
-    const int lz = __clzll((long long)a);       // >= 1: |t| < 2^63
-    const unsigned long long m = (a << (lz - 1)) + 0x200u;      // leading bit at 62
-    // leading bit 2^(63 - lz) of t: exponent unit + 63 - lz, one of it from the
-    // leading bit itself (bit 20 of the high word)
-    const unsigned hi = (unsigned)(m >> 42) + ((unsigned)(unit + 63 - lz + 1023 - 1) << 20);
-    return __hiloint2double((int)(hi | ((unsigned)s & 0x80000000u)), (int)(unsigned)(m >> 10));
-}
-
 // The sums as doubles, for warps that leave the integer form after all.
 __device__ __forceinline__ void quad_to_double(QuadSums &s)
 {

@@ -69,7 +69,7 @@ cudaError_t Launchers<D, Codec>::step_fd(qlbm_ctx *h, bool odd)
             cudaThreadExchangeStreamCaptureMode(&mode);
         }
         FixConst fc;
-        if (h->fd_rho && make_fix_const(h->hc, h->dt / h->tau, &fc)) {
+        if (h->fd_rho && make_fix_const(h->hc, h->dt / h->tau, false, &fc)) {
             FdOut o{};
             o.rho = static_cast<DQuad *>(h->fd_rho);
             o.flags = h->flags;
