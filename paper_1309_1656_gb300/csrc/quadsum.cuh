@@ -420,7 +420,13 @@ k_negative_eq(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Codec c
         double sq = c == 0 ? 0.0 : M * M;
         sq += __shfl_xor_sync(all, sq, 1, 4);
         sq += __shfl_xor_sync(all, sq, 2, 4);
-        const bool polar = M * M < sq;      // of lane 0: n < |S|
+        // of lane 0: n < |S|, by the root where the squares are close (pure
+        // states: it halves the squares' rounding, and a zero eigenvalue does
+        // not count; ~20 double-precision instructions elsewhere too if taken
+        // always)
+        const double MM = M * M;
+        bool polar = MM < sq;
+        if (c == 0 && abs(__double2hiint(MM) - __double2hiint(sq)) <= 1) polar = M < sqrt(sq);
         fx_each_h<D>(cf, [&](int q, long long h) {
             if (h < 0 || (polar && h > 0)) m |= 1u << q;
         });

@@ -116,3 +116,27 @@ def test_device_mask_and_bench_workload(q, oracle_mod):
     # smooth near-equilibrium fields (|u| <= 0.05, eps = eps0): every P_i
     # stays near 1 and |S| << n, so none is negative-definite
     assert c_host == 0
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
+@pytest.mark.parametrize("d,dims", [(2, (61, 9, 1)), (3, (17, 6, 5))])
+def test_pure_states_compare_n_with_the_root(q, prec, d, dims):
+    # |S| = n up to rounding along random axes: every direction of a site is
+    # flagged exactly where n < sqrt(S.S) in double, n and S being the sums
+    # that qlbm_moments returns (all P_i > 0: u = 0, eps the reference's)
+    N = int(np.prod(dims))
+    rng = np.random.default_rng(71)
+    axis = rng.normal(size=(3, N))
+    axis /= np.linalg.norm(axis, axis=0)
+    n = rng.uniform(0.5, 1.5, N)
+    n[::3] = 1.0
+    axis[:, ::5] = [[0.0], [0.0], [1.0]]
+    with q.Lattice(d, dims, 0.8, 1.0, precision=prec) as lat:
+        lat.init_equilibrium(np.concatenate([n[None], n * axis]), np.zeros((d, N)), None)
+        r, u, eps = lat.moments()
+        mask = np.zeros(N, dtype=np.uint32)
+        count = q.qlbm_negative_eq_count(lat.h, mask)
+    polar = r[0] < np.sqrt(r[1] * r[1] + (r[2] * r[2] + r[3] * r[3]))
+    assert polar.any() and not polar.all()
+    assert np.array_equal(mask, np.where(polar, (1 << (9 if d == 2 else 19)) - 1, 0))
+    assert count == int(polar.sum()) * (9 if d == 2 else 19)
