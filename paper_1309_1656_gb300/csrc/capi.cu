@@ -516,7 +516,11 @@ int64_t qlbm_time(qlbm_handle h) { return h ? h->t : -1; }
 int qlbm_sync(qlbm_handle h)
 {
     if (!valid(h)) return fail(h, QLBM_ERR_INVALID_ARG, "qlbm_sync: bad handle");
-    return check_flags(h);
+    // a copy, not k_report: this call waits for work that is there and launches
+    // none, so the handle's device need not be the calling thread's current one
+    CK(h, cudaMemcpyAsync(&h->report->flags, h->flags, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
+    return report_flags(h);
 }
 
 int qlbm_moments(qlbm_handle h, double *rho4, double *u, double *eps, int ptr_kind)
