@@ -68,10 +68,11 @@ __global__ void k_report(const unsigned *flags, const unsigned long long *counte
 
 namespace {
 
-// Report slots come from pages of 32 (allocating host memory that the device
-// can write takes ~0.1 ms, a tenth of creating a small handle).  A page goes
-// when its last slot is returned, but for one; the mutex covers handles made
-// and destroyed by several threads.
+// Report slots come from pages of 32, shared by the handles that are alive
+// (allocating host memory that the device can write takes ~0.1 ms).  A page
+// goes when its last slot is returned: none outlives the handles, as
+// cudaDeviceReset would free it underneath the next one.  The mutex covers
+// handles made and destroyed by several threads.
 struct ReportPage {
     HostReport *slots;
     unsigned used;      // bit i: slot i is taken
@@ -119,7 +120,7 @@ void give_report(HostReport *r)
         for (int i = 0; i < 32; ++i)
             if (report_slot(report_pages[k], i) == r) {
                 report_pages[k].used &= ~(1u << i);
-                if (!report_pages[k].used && report_pages.size() > 1) {
+                if (!report_pages[k].used) {
                     cudaFreeHost(report_pages[k].slots);
                     report_pages.erase(report_pages.begin() + (long)k);
                 }
