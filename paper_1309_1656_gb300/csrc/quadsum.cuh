@@ -22,16 +22,19 @@ namespace qlbm {
 
 // One stored value as the integer sums take it: key() orders magnitudes, its
 // bits from KEY_EXP on are the biased exponent (bias BIAS); align() gives the
-// value in units of 2^(e - BIAS - 57) for a largest exponent e.
+// value in units of 2^(e - BIAS - 57) for a largest exponent e >= MIN_EXP.  A
+// component below that is taken times 2^LIFT (exact, subnormals included),
+// where LIFT is not 0.
 template <class Codec> struct QuadValue;
 template <> struct QuadValue<CodecF64> {
     using Raw = unsigned long long;
-    static constexpr int KEY_EXP = 20, BIAS = 1023, MIN_EXP = kFxMinExp, MAX_EXP = kFxMaxExp;
+    static constexpr int LIFT = 0, KEY_EXP = 20, BIAS = 1023, MIN_EXP = kFxMinExp, MAX_EXP = kFxMaxExp;
     static __device__ __forceinline__ Raw load(const CodecF64 &, const DQuad *p, int c)
     {
         return reinterpret_cast<const unsigned long long *>(p)[c];
     }
     static __device__ __forceinline__ unsigned key(Raw w) { return (unsigned)(w >> 32) & 0x7fffffffu; }
+    static __device__ __forceinline__ Raw lift(Raw w) { return w; }
     static __device__ __forceinline__ long long align(Raw w, int e) { return fx_align((unsigned)(w >> 32), (unsigned)w, e); }
     static __device__ __forceinline__ double value(const CodecF64 &, Raw w, int, int)
     {
@@ -47,10 +50,12 @@ __device__ __forceinline__ long long fx_align_float(unsigned b, int e)
     const long long s = (long long)((int)b >> 31);
     return (x ^ s) - s;
 }
+__device__ __forceinline__ unsigned fx_lift_float(unsigned b) { return __float_as_uint(__uint_as_float(b) * 0x1p96f); }
 struct QuadValueFloat {
     using Raw = unsigned;
-    static constexpr int KEY_EXP = 23, BIAS = 127, MIN_EXP = 66, MAX_EXP = 127 + 90;
+    static constexpr int LIFT = 96, KEY_EXP = 23, BIAS = 127, MIN_EXP = 66, MAX_EXP = 127 + 90;
     static __device__ __forceinline__ unsigned key(Raw w) { return w & 0x7fffffffu; }
+    static __device__ __forceinline__ Raw lift(Raw w) { return fx_lift_float(w); }
     static __device__ __forceinline__ long long align(Raw w, int e) { return fx_align_float(w, e); }
 };
 template <> struct QuadValue<CodecF32> : QuadValueFloat {
@@ -75,12 +80,13 @@ template <> struct QuadValue<CodecF16Dev> : QuadValueFloat {
 };
 template <> struct QuadValue<CodecDF> {
     using Raw = uint2;      // hi, lo
-    static constexpr int KEY_EXP = 23, BIAS = 127, MIN_EXP = 66, MAX_EXP = 127 + 90;
+    static constexpr int LIFT = 96, KEY_EXP = 23, BIAS = 127, MIN_EXP = 66, MAX_EXP = 127 + 90;
     static __device__ __forceinline__ Raw load(const CodecDF &k, const float4 *p, int c)
     {
         return make_uint2(reinterpret_cast<const unsigned *>(p)[c], reinterpret_cast<const unsigned *>(p + k.lo)[c]);
     }
     static __device__ __forceinline__ unsigned key(Raw w) { return max(w.x & 0x7fffffffu, w.y & 0x7fffffffu); }
+    static __device__ __forceinline__ Raw lift(Raw w) { return make_uint2(fx_lift_float(w.x), fx_lift_float(w.y)); }
     static __device__ __forceinline__ long long align(Raw w, int e) { return fx_align_float(w.x, e) + fx_align_float(w.y, e); }
     static __device__ __forceinline__ double value(const CodecDF &k, Raw w, int comp, int cls)
     {
@@ -130,7 +136,17 @@ __device__ __forceinline__ QuadSums quad_sums(const Planes<typename Codec::S, La
     unsigned mx = 0u;
 #pragma unroll
     for (int q = 0; q < Q; ++q) mx = max(mx, V::key(w[q]));
-    const int em = (int)(mx >> V::KEY_EXP);
+    int em = (int)(mx >> V::KEY_EXP), lifted = 0;
+    if (V::LIFT && mx && em < V::MIN_EXP && !(Codec::DEV && c == 0)) {
+        lifted = V::LIFT;
+        mx = 0u;
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            w[q] = V::lift(w[q]);
+            mx = max(mx, V::key(w[q]));
+        }
+        em = (int)(mx >> V::KEY_EXP);
+    }
     int e = em;
     bool ok = em >= V::MIN_EXP && em <= V::MAX_EXP;
     if (Codec::DEV && c == 0) {
@@ -142,7 +158,7 @@ __device__ __forceinline__ QuadSums quad_sums(const Planes<typename Codec::S, La
         ok = true;
     }
     o.fine = __all_sync(0xffffffffu, ok);
-    o.unit = e - V::BIAS - 57;
+    o.unit = e - V::BIAS - 57 - lifted;
     if (o.fine) {
         long long X[Q];
 #pragma unroll
@@ -162,6 +178,13 @@ __device__ __forceinline__ QuadSums quad_sums(const Planes<typename Codec::S, La
             if (cy<D>(q)) o.dJ[1] += cy<D>(q) * v;
             if (cz<D>(q)) o.dJ[2] += cz<D>(q) * v;
             if (cnorm2<D>(q)) o.dE += cnorm2<D>(q) * v;
+        }
+        if (lifted) {
+            constexpr double down = V::LIFT ? 0x1p-96 : 1.0;
+            o.dM *= down;
+            o.dE *= down;
+#pragma unroll
+            for (int a = 0; a < 3; ++a) o.dJ[a] *= down;
         }
     }
     return o;
@@ -233,20 +256,31 @@ __device__ __forceinline__ void site_sums(const Planes<typename Codec::S, Lattic
     float f[4][Q];
     gather<D, Codec, SWAPPED>(pl, g, si, codec, f[0], f[1], f[2], f[3]);
     o.fine = true;
+    bool lifted[4];
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
         unsigned mx = 0u;
 #pragma unroll
         for (int q = 0; q < Q; ++q) mx = max(mx, V::key(__float_as_uint(f[c][q])));
-        const int em = (int)(mx >> V::KEY_EXP);
+        int em = (int)(mx >> V::KEY_EXP);
         int e = V::BIAS - 1;
+        lifted[c] = c && mx && em < V::MIN_EXP;
         if (c == 0) {
             o.fine = o.fine && em <= e;
         } else if (mx) {
+            if (lifted[c]) {
+                mx = 0u;
+#pragma unroll
+                for (int q = 0; q < Q; ++q) {
+                    f[c][q] *= 0x1p96f;
+                    mx = max(mx, V::key(__float_as_uint(f[c][q])));
+                }
+                em = (int)(mx >> V::KEY_EXP);
+            }
             o.fine = o.fine && em >= V::MIN_EXP && em <= V::MAX_EXP;
             e = em;
         }
-        o.unit[c] = e - V::BIAS - 57;
+        o.unit[c] = e - V::BIAS - 57 - (lifted[c] ? V::LIFT : 0);
         if (c == 0) {
             long long X[Q];
 #pragma unroll
@@ -275,6 +309,7 @@ __device__ __forceinline__ void site_sums(const Planes<typename Codec::S, Lattic
                 if (cz<D>(q)) o.dJ[2] += cz<D>(q) * v;
                 if (cnorm2<D>(q)) o.dE += cnorm2<D>(q) * v;
             }
+            if (lifted[c]) o.dM[c] *= 0x1p-96;
         }
     }
 }

@@ -123,3 +123,27 @@ def test_initial_equilibrium(q, prec, d, dims):
     slack = np.zeros_like(want)
     slack[:, 0] = 2.0 ** -47 * np.abs(rho4[0])
     assert np.all(np.abs(stored.astype(LD) - want) <= 0.501 * ulp + slack)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "df64", "fp32"])
+@pytest.mark.parametrize("d,dims", [(2, (33, 5, 1)), (3, (17, 3, 4))])
+def test_tiny_spins(q, prec, d, dims):
+    # spins from 2^-50 down to single precision's subnormals and to zero, each
+    # component a size of its own, and now and then a site summed in double
+    rng = np.random.default_rng(61)
+    st = fields.random_populations(d, dims, seed=13)
+    N = st.shape[2]
+    for c in (1, 2, 3):
+        st[:, c] *= 2.0 ** -rng.integers(50, 150, N)
+    st[:, 1, ::11] = 0.0
+    if N > 40:
+        st[0, 0, ::40] = -3.0
+    with q.Lattice(d, dims, 0.8, 1.0, precision=prec) as lat:
+        lat.set_state(st)
+        W = lat.get_state().astype(LD)
+        r, u, eps = lat.moments()
+        total = lat.conserved()
+    assert np.all(np.abs(r - W.sum(0)) <= TOL * np.abs(W).sum(0))
+    if prec != "fp32":      # (its global sums are formed in double-float, to single precision's range)
+        for c in (1, 2, 3):
+            assert abs(total[c] - W[:, c].sum() / N) <= 4 * TOL * np.abs(W[:, c]).sum() / N
