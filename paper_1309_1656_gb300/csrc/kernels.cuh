@@ -19,6 +19,7 @@ struct InitConsts {
     double xi, K, c, inv_mc2, c3, c4, c5, eps0, beta0;
     double w[3];
     double rxi, rK, umax;   // 2^64 / xi, 2^60 / K, 3/8 xi
+    bool rest;              // beta0 eps0 is c to the last bit
 };
 
 template <int D>

@@ -75,6 +75,7 @@ inline InitConsts make_init(const qlbm_ctx *h)
     ic.rxi = 0x1p64 / k.xi;
     ic.rK = 0x1p60 / k.K;
     ic.umax = 0.375 * k.xi;
+    ic.rest = k.beta0 * k.eps0 == k.c;
     return ic;
 }
 
