@@ -381,11 +381,12 @@ inline long long fx_one_minus(double omega)
 // Host: the constants, false where they leave the form's range (then the
 // double-precision kernel steps the lattice).  normalise: h_i for omega 2^k in
 // [1/2, 1) instead of a smaller omega, so that it keeps its digits (for the
-// update in double, which takes it in units of 2^-(62 + k)).
+// update in double, which takes it in units of 2^-(62 + k): from 2^-900 on, so
+// that h_i's last place is a normal double).
 inline bool make_fix_const(const HostConsts &k, double omega, bool normalise, FixConst *o)
 {
     *o = FixConst{};
-    if (!(omega > 0.0 && omega <= 2.0)) return false;
+    if (!(omega >= 0x1p-900 && omega <= 2.0)) return false;
     o->h_unit = -62;
     if (normalise && omega < 0.5) {
         int e;

@@ -1,6 +1,7 @@
 // Host entry points to the device headers' arithmetic (functions compiled for
 // both sides), for the checks that need no GPU: loaded by
 // test_host_arithmetic.py.
+#include "../paper_1309_1656_gb300/csrc/consts.cu"
 #include "../paper_1309_1656_gb300/csrc/fdparams.cuh"
 #include "../paper_1309_1656_gb300/csrc/fix64.cuh"
 
@@ -29,3 +30,13 @@ extern "C" double fd_table_offset(float x) { return (double)x - (FD_PX0 + 0.125 
 
 // 1 - omega as the FP64 step's constants hold it (q62).
 extern "C" long long one_minus_omega(double omega) { return fx_one_minus(omega); }
+
+// Smallest exponent of a coefficient h_i that is not zero, for the update in
+// double of a D2Q9 or D3Q19 step at `omega`; 0 where the form is not taken.
+extern "C" int least_coefficient_exponent(int d, double omega)
+{
+    HostConsts k;
+    FixConst fc;
+    if (compute_constants(d, 1.0, &k) != 0) return 1;
+    return make_fix_const(k, omega, true, &fc) ? fc.h_unit : 0;
+}

@@ -142,3 +142,11 @@ def test_small_spin_components_in_a_field(q, d, dims, site, axis, omega):
     if site:
         B = B * rng.uniform(0.5, 1.5, N)
     run(q, d, dims, omega, st, field=B)
+
+
+# at an omega this small the step leaves the state as it is, but for streaming
+@pytest.mark.parametrize("tau", [1e200, 1e270, 1e290, 1e300])
+@pytest.mark.parametrize("prec", ["fp64", "fp64df"])
+@pytest.mark.parametrize("d,dims", [(2, (21, 5, 1)), (3, (9, 5, 3))])
+def test_endless_relaxation(q, d, dims, prec, tau):
+    run(q, d, dims, 1.0 / tau, one_outweighs(d, dims, 0.1), prec=prec)

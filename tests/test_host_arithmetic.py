@@ -71,3 +71,11 @@ def test_one_minus_omega_stays_within_64_bits(tmp_path):
     lib = compile_host(tmp_path, "-fPIC,-fsanitize=signed-integer-overflow,-fsanitize-undefined-trap-on-error")
     code = "import ctypes; f = ctypes.CDLL(%r).one_minus_omega; [f(ctypes.c_double(w)) for w in %r]" % (lib, OMEGAS)
     assert subprocess.run([sys.executable, "-c", code]).returncode == 0
+
+
+@pytest.mark.parametrize("d", [2, 3])
+def test_coefficients_of_a_tiny_omega_are_normal_doubles(host, d):
+    # (their words are put together in integers; below, the step is in double)
+    for k in range(0, 1075):
+        assert host.least_coefficient_exponent(d, ctypes.c_double(2.0**-k)) in [0] + list(range(-1022, -61))
+    assert all(host.least_coefficient_exponent(d, ctypes.c_double(w)) for w in (2.0**-900, 1e-9, 0.5, 1.0, 2.0))
