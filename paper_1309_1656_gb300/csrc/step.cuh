@@ -40,8 +40,8 @@ template <class S, int Q> struct Planes {
 // (let_next_start; at the kernels' start instead, the successor's waiting
 // blocks get in the way: 64 x 64 FP64 3.07 us per step, D3Q19 32^3 FP32 4.9).
 // Without effect next to other work.  Per step, before -> after: D2Q9 64^2
-// FP64 2.64 -> 2.25 us, D2Q9 256^2 FP64 10.1 -> 9.7, D3Q19 128^3 FP16 102.8 ->
-// 100.0, FP32 186.6 -> 184.3.
+// FP64 2.64 -> 2.25 us, FP16 2.0 -> 1.6, D2Q9 256^2 FP64 10.1 -> 9.7, D2Q9
+// 1501 x 777 DF64 114.3 -> 111.4.
 __device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -280,7 +280,10 @@ k_step_aa_rows(const Planes<typename Codec::S, Lattice<D>::Q> pl, Grid g, Coll<t
         }
         flag |= Codec::template collide<D>(f, sx, sy, sz, k);
         apply_field<D, FIELD, R>(sx, sy, sz, k, cur.s);
-        if (row + 1 == rend) let_next_start();
+        // (in 3D the check costs the row loop more than the early start gives:
+        // 128^3 101.8 us per step instead of 100.4, 64^3 12.2 instead of 11.9,
+        // 32^3 3.1 instead of 3.0; D2Q9 64^2 1.6 with it, 2.0 without)
+        if (D == 2 && row + 1 == rend) let_next_start();
         // store addresses recomputed from g.zero (see k_step_aa)
         const int so = cur.s + g.zero;
 #pragma unroll
