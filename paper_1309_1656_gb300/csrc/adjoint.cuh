@@ -30,60 +30,6 @@ namespace qlbm {
 
 constexpr int kAdjBlock = 128;
 
-// Forward moments of one site in either representation (DEV: deviations
-// d_i = f_i - w_i), as needed by the adjoint.
-template <int D, typename R, bool DEV> struct FwdSite {
-    R n, dn, Sx, Sy, Sz, jx, jy, jz, e2n, jj, a2;
-};
-
-template <int D, typename R, bool DEV>
-__device__ __forceinline__ FwdSite<D, R, DEV> forward_moments(const R *f, const R *sx, const R *sy,
-                                                             const R *sz, const Coll<R> &k)
-{
-    constexpr int Q = Lattice<D>::Q;
-    FwdSite<D, R, DEV> m;
-    R sn = R(0), Sx = R(0), Sy = R(0), Sz = R(0), Jx = R(0), Jy = R(0), Jz = R(0), E = R(0);
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-        sn += f[q];
-        Sx += sx[q];
-        Sy += sy[q];
-        Sz += sz[q];
-        Jx += cx<D>(q) * f[q];
-        Jy += cy<D>(q) * f[q];
-        Jz += cz<D>(q) * f[q];
-        E += cnorm2<D>(q) * f[q];
-    }
-    m.dn = DEV ? sn : sn - R(1);
-    m.n = DEV ? R(1) + sn : sn;
-    const R rn = R(1) / m.n;
-    m.Sx = Sx;
-    m.Sy = Sy;
-    m.Sz = Sz;
-    m.jx = Jx * rn;
-    m.jy = Jy * rn;
-    m.jz = Jz * rn;
-    m.jj = m.jx * m.jx + m.jy * m.jy + m.jz * m.jz;
-    R de;   // E2/n - S2
-    if (DEV) {
-        de = (E - k.S2 * sn) * rn;
-        m.e2n = k.S2 + de;
-    } else {
-        m.e2n = E * rn;
-        de = m.e2n - k.S2;
-    }
-    // K (E2/n - |j|^2) - c = K (de - |j|^2)  (c = K S2)
-    m.a2 = k.K * (de - m.jj) * k.inv_mc2;
-    return m;
-}
-
-template <int D, typename R, bool DEV>
-__device__ __forceinline__ R P1_of(const FwdSite<D, R, DEV> &m, const Coll<R> &k, int q)
-{
-    const R t = cx<D>(q) * m.jx + cy<D>(q) * m.jy + cz<D>(q) * m.jz;
-    return m.a2 * (k.K * cnorm2<D>(q) - k.c) + t * (k.c3 + k.c4 * t) + k.c5 * m.jj;
-}
-
 template <typename R>
 __device__ __forceinline__ double block_sum_double(double v)
 {

@@ -102,13 +102,6 @@ __device__ __forceinline__ int nb_at(const NbOff &o, int s, int ex, int ey, int 
 {
     return s + nb_axis(ex, o.xp, o.xm) + nb_axis(ey, o.yp, o.ym) + nb_axis(ez, o.zp, o.zm);
 }
-// Indices of s + e and s - e.
-__device__ __forceinline__ void nb_pair(const NbOff &o, int s, int ex, int ey, int ez, int &sp, int &sm)
-{
-    sp = s + nb_axis(ex, o.xp, o.xm) + nb_axis(ey, o.yp, o.ym) + nb_axis(ez, o.zp, o.zm);
-    sm = s + nb_axis(ex, o.xm, o.xp) + nb_axis(ey, o.ym, o.yp) + nb_axis(ez, o.zm, o.zp);
-}
-
 // Gathers the b populations of site si at the current time, in arithmetic
 // type R.  SWAPPED selects the reading pattern of a buffer last written by
 // an even step.
