@@ -38,10 +38,12 @@
 // Blocks of two warps (a 64 x 64 lattice reaches every SM); 16 warps per SM
 // at 128 registers for D3Q19 (20 at 96 spill: 548 us).
 //
-// Measured (double-precision kernel -> this one): D3Q19 128^3 1485 -> 507 us,
-// D2Q9 2048^2 1512 -> 527 us, D2Q9 64^2 8.3 -> 2.65 us and 2048 x 2 9.2 -> 2.7
-// us per step.  Now bound by issue and the integer and multiply pipes
-// together (60-64 % each, ~1390 instructions per warp of 8 sites).
+// Measured (double-precision kernel -> this one), updated in integers: D3Q19
+// 128^3 1485 -> 504 us, D2Q9 2048^2 1512 -> 527 us, D2Q9 64^2 8.2 -> 2.3 us; in
+// double: 1485 -> 659 us, 1516 -> 594 us, 64^2 2.9 and 2048 x 2 9.0 -> 2.8 us per
+// step.  The former is bound by issue (57 % of the cycles), the integer pipe (62 %
+// busy), the multiply pipe (60 %) and the conversions (51 %) together, at 1360
+// instructions per warp of 8 sites; the latter by the double pipe.
 #pragma once
 
 #include <math.h>
@@ -617,19 +619,22 @@ enum : int { FIX_EVEN = 0, FIX_ODD = 1, FIX_PUSH = 2 };
 // adds each.  The fixed-point update errs by up to 1.3 x 2^-56 of the
 // component's largest value whatever omega is, the double step by a few 2^-53
 // of omega h M and by 2^-54 of the result: for a population much smaller than
-// the largest the double step is the better one where omega is small.  Root
-// mean square errors of populations between 2^-5 and 2^-4 of the largest, in
-// 2^-53 of themselves, over random sites (D3Q19; fixed point, double step):
-// omega = 1.25: 0.9, 4.4; 0.5: 0.9, 1.8; 0.1: 0.9, 0.5; 0.01: 0.9, 0.4, and in
-// proportion below; where one population outweighs all others the double step
-// gains on it from 0.7 down.  In double D3Q19 128^3 takes 660 us instead of
-// 505, with a field 1436 instead of 702, D2Q9 64^2 2.9 instead of 2.3 (the
-// double pipe; 1485, 2207 and 8.3 with everything in double).  QLBM_FP64_DF
-// with a field, stated to 1e-14 of the largest, keeps the fixed-point update
-// further down.
+// the largest the double step is the better one where omega is small.  The
+// line lies where its errors reach the double step's on such populations, in
+// 2^-53 of the terms of each result (largest and root mean square; fixed point,
+// double step; one population of 1 and the others near 1e-6, D2Q9): omega =
+// 0.75: 1.5 0.35, 2.3 0.51; 0.65: 2.0 0.42, 2.2 0.51; 0.6: 2.2 0.46, 2.1 0.51;
+// 0.5: 2.5 0.52, 2.0 0.51; with a field 0.7: 1.7
+// 0.22, 2.0 0.28; 0.65: 2.0 0.23, 1.7 0.28.  (Populations near equilibrium: 0.4:
+// 2.9 0.44, 3.3 0.65.)  In double D3Q19 128^3 takes 659 us instead of 504, with a
+// field 1436 instead of 702, D2Q9 64^2 2.9 instead of 2.3 (the double pipe; 1485,
+// 2207 and 8.2 with everything in double).  The change h M - omega W in
+// integers at omega's own scale and one addition in double instead was as
+// exact and slower (749 us; 64^2 2.96).  QLBM_FP64_DF with a field, stated to
+// 1e-14 of the largest, keeps the fixed-point update further down.
 inline double fix_double_below(int prec, int field)
 {
-    return prec == QLBM_FP64 || field == FIELD_NONE ? 0.75 : 0.0625;
+    return field == FIELD_NONE ? 0.65 : prec == QLBM_FP64 ? 0.7 : 0.0625;
 }
 template <int D, int MODE, bool FD, int FIELD, bool DBL>
 __global__ void __launch_bounds__(kFixBlock, D == 3 ? 8 : 14)

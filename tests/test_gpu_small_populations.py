@@ -9,9 +9,9 @@ absolute terms of P_i and T = |v| + omega w_i A_i |M|, a step in double errs by
 2^-53 of: v, the product omega h M and their sum once each, and the
 coefficients' own roundings, at most ~4 of omega w_i A_i |M|: 8 x 2^-53 T.  Sums
 M of populations of one sign err by a few 2^-53 of M more: 16 x 2^-53 T in all.
-The fixed-point form (omega from 3/4 on) errs by 1.3 x 2^-56 of the component's
+The fixed-point form (omega from 0.65 on) errs by 1.3 x 2^-56 of the component's
 largest value at the site, which is at most b times |M| for populations of one
-sign: within the same bound there, as omega w_i A_i >= 0.75 / 36 x A_i and A_i
+sign: within the same bound there, as omega w_i A_i >= 0.65 / 36 x A_i and A_i
 is at least 1.  A field's rotation R mixes the bounds: sum_b |R_ab| T_b, and
 8 x 2^-53 sum_b |R_ab| max |W_b| for the fixed-point form's common alignment of
 what it mixes."""
@@ -115,7 +115,7 @@ def one_outweighs(d, dims, small):
     return st
 
 
-@pytest.mark.parametrize("omega", [1.9, 1.25, 0.75, 0.7, 0.5, 0.1, 0.01, 0.001])
+@pytest.mark.parametrize("omega", [1.9, 1.25, 0.75, 0.66, 0.5, 0.1, 0.01, 0.001])
 @pytest.mark.parametrize("small", [1e-2, 1e-6, 1e-12])
 @pytest.mark.parametrize("d,dims", [(2, (21, 5, 1)), (3, (9, 5, 3))])
 def test_small_populations(q, d, dims, small, omega):
