@@ -230,8 +230,8 @@ def job_mlups(ws, sites_per_rank, steps, seconds):
 # Step kernel per precision, and what bounds it when it is not HBM bandwidth.
 STEP_KERNEL = {"fp32": "k_step_aa<%d, CodecF32>", "fp16dev": "k_step_aa_rows<%d, CodecF16Dev>",
                "fp64": "k_step_fix<%d>", "fp64df": "k_step_fix<%d>", "df64": "k_step_aa_df2<%d>"}
-STEP_LIMIT = {"fp64": "issue: ~1390 integer instructions per warp of 8 sites (fixed-point products, alignment), "
-                      "integer and multiply pipes 60-64 % busy",
+STEP_LIMIT = {"fp64": "issue: 1360 instructions per warp of 8 sites (fixed-point products, alignment); 57 % of "
+                      "issue slots, integer pipe 62 %, multiply pipe 60 %, conversions 51 % busy",
               "fp64df": "issue: the FP64 kernel"}
 
 

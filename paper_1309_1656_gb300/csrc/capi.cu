@@ -862,8 +862,9 @@ int qlbm_set_magnetic_field_array(qlbm_handle h, double mu, const double *B, int
     if (!(mu == mu) || !(fabs(mu) < 1e300))
         return fail(h, QLBM_ERR_INVALID_ARG, "qlbm_set_magnetic_field_array: mu must be finite");
     const int64_t N = h->g.N;
-    // quaternions as doubles for the 64-bit precisions (the double-float
-    // steps split them), as floats for the single-precision arithmetic
+    // quaternions as doubles for the 64-bit precisions (double-float storage
+    // forms a site's rotation from them in double), as floats for the
+    // single-precision arithmetic
     const bool dbl = h->prec == QLBM_FP64 || h->prec == QLBM_FP64_DF || h->prec == QLBM_DF64;
     const size_t vb = dbl ? sizeof(DQuad) : sizeof(float4);
     if (!h->qfield) CK(h, cudaMalloc(&h->qfield, (size_t)N * vb));

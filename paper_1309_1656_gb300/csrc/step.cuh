@@ -102,6 +102,7 @@ __device__ __forceinline__ int nb_at(const NbOff &o, int s, int ex, int ey, int 
 {
     return s + nb_axis(ex, o.xp, o.xm) + nb_axis(ey, o.yp, o.ym) + nb_axis(ez, o.zp, o.zm);
 }
+
 // Gathers the b populations of site si at the current time, in arithmetic
 // type R.  SWAPPED selects the reading pattern of a buffer last written by
 // an even step.
